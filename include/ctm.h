@@ -141,29 +141,23 @@ typedef struct {
 /* Launch-shape tuning of a context (no effect on results).  Not described
  * by the paper: these are choices of this implementation's kernels. */
 typedef struct {
-    int32_t match_threads;  /* matching CTA size: 128 or 256 threads                    */
-    int32_t strip_cols;     /* width, in codes, of the staged strip of one column chunk
-                               of a block: a multiple of 8, at least the larger
-                               disparity range + 2; larger values mean fewer chunks
-                               and more shared memory per CTA                         */
+    int32_t match_threads;  /* per-box and two-pass matchers: CTA size, 128 or 256 threads */
+    int32_t strip_cols;     /* per-box and two-pass matchers: width, in codes, of the staged
+                               strip of one column chunk of a block: a multiple of 8, at
+                               least the larger disparity range + 2; larger values mean
+                               fewer chunks and more shared memory per CTA            */
     int32_t census_mode;    /* region-of-interest census (5x5, 7x7, 9x7 windows): 0 =
                                integer multiply-add compares, 4 CTAs per SM; 1 = the
                                same, 3 CTAs per SM; 2 = packed fp16 compares with
                                saturation, 4 CTAs per SM                              */
-    int32_t queue_rounds;   /* fused matcher: 1 = the first blocks of a launch go out in
-                               per-SM rounds (every SM one block of each round; the
-                               queue runs from the largest blocks down), 0 = one
-                               dynamic queue                                          */
-    int32_t match_mode;     /* 0: fused matcher (one CTA runs both passes of a block);
-                               1: two-pass pipelined matcher (a forward kernel, then a
-                               backward kernel; each CTA loads its next block while it
-                               scans the current one)                                 */
-    int32_t split_ways;     /* fused matcher only: 0 = split every block's candidate range
-                               into two (block, disparity-chunk) tiles when the queue
-                               holds fewer than about 0.6 blocks per resident CTA and
-                               the CLOSE range has at least 128 candidates; 1 = never
-                               split; 2, 4 or 8 = always split into that many chunks.
-                               Splitting needs one vertical offset (dy_min == dy_max) */
+    int32_t queue_rounds;   /* 0 or 1; accepted and kept, without effect (no matcher hands
+                               blocks out in rounds any more)                          */
+    int32_t match_mode;     /* 0: tensor-core matcher (both passes of a block as products of
+                               e2m1 operands, exact; tcgen05); 1: two-pass pipelined
+                               matcher (a forward kernel, then a backward kernel; each CTA
+                               loads its next block while it scans the current one)    */
+    int32_t split_ways;     /* 0, 1, 2, 4 or 8; accepted and kept, without effect (no
+                               matcher splits a block's candidate range any more)      */
 } ctm_tuning;
 
 /* Counters of the last match call (ctm_get_stats). */
@@ -377,9 +371,9 @@ int ctm_get_tuning(const ctm_ctx *ctx, ctm_tuning *out);
 int ctm_set_tuning(ctm_ctx *ctx, const ctm_tuning *t);
 
 /* Autotuner: runs the batch of ctm_match_batch (same arguments, no debug
- * output) under candidate tunings -- every matching CTA size x strip width,
- * for each matcher, then each census variant, rounds on and off and automatic
- * or no disparity-chunk tiles around the best so far --
+ * output) under candidate tunings -- the tensor-core matcher, the two-pass
+ * matcher at every CTA size x strip width, then each census variant around the
+ * best so far --
  * timing `reps` calls of each with CUDA events after one warm-up call, keeps
  * the fastest in the context and returns it in *best (and its time per call,
  * in ms, in *best_ms; either may be NULL).  The outputs are written by every
@@ -398,13 +392,13 @@ int ctm_autotune(ctm_ctx *ctx, const ctm_frame *frames_dev, const int32_t *count
 int ctm_probe_int_rate(int kind, int iters, double *ops_per_clk_per_sm);
 
 /* Fault injection for tests (no counterpart in the paper): arms ctx so that the
- * next match call on it that launches the fused persistent matcher directly
+ * next match call on it that launches the tensor-core matcher directly
  * (ctm_match_boxes, ctm_match_batch with use_graph = 0, ctm_match_batch_host;
  * tuning match_mode 0; not a graph replay, not the plain per-box path) has its
- * CTA that takes the queue's first block (or first tile) announce a strip copy
- * on its mbarrier without issuing it.  That CTA's bounded wait then expires (about 1 s, then about 1 s more for the
- * copies in flight, of which there are none), it records the error and stops;
- * the other CTAs finish the queue.  The call's outputs follow the CTM_ETIMEOUT
+ * worker that takes the queue's first block withhold the completion signal of
+ * that block's products.  The worker's bounded wait then expires (about 1 s, then
+ * about 1 s more), it records the error, lets its products end and stops;
+ * the other workers finish the queue.  The call's outputs follow the CTM_ETIMEOUT
  * rule above, and ctm_match_batch_host returns CTM_ETIMEOUT.  The arming is
  * consumed by that one call; the context stays usable.  No GPU fault is
  * involved.  Errors: CTM_EINVAL (null ctx). */

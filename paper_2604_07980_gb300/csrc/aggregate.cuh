@@ -121,4 +121,35 @@ __device__ __forceinline__ void write_block(const MatchArgs &a, int box, int slo
     if (a.dbg.blocks) a.dbg.blocks[(long long)box * (a.p.grid_g * a.p.grid_g) + slot] = rec;
 }
 
+// Block record from the two passes' results (Eq. subpixel on the forward costs
+// around d_f, consistency |d_b - d_f| <= fb_tol); g: the block's sampling record.
+__device__ __forceinline__ void write_record(const MatchArgs &a, const BlockGeom &g, int d_f, int dy_f, int d_b,
+                                             int dy_b, int s_m, int s_0, int s_p)
+{
+    ctm_block rec;
+    rec.n_pts = g.nx * g.ny;
+    rec.n_valid = g.n_valid;
+    rec.flags = CTM_BLK_PRESENT;
+    rec.d_f = d_f;
+    rec.dy_f = dy_f;
+    rec.d_b = d_b;
+    rec.dy_b = dy_b;
+    rec.s_m = s_m;
+    rec.s_0 = s_0;
+    rec.s_p = s_p;
+    if (rec.d_f == g.dmin || rec.d_f == g.dmax) {
+        rec.d_sub = (float)rec.d_f;
+        rec.flags |= CTM_BLK_SUBPIX_CLAMPED;
+    } else {
+        // Eq. subpixel
+        const float num = (float)(rec.s_p - rec.s_m);
+        const float den = __fmul_rn(2.0f, (float)(rec.s_p + rec.s_m - 2 * rec.s_0));
+        rec.d_sub = den == 0.0f ? (float)rec.d_f : __fsub_rn((float)rec.d_f, __fdiv_rn(num, den));
+    }
+    rec.d_full = __fmul_rn(rec.d_sub, (float)g.k);
+    const int dxv = abs(rec.d_b - rec.d_f);
+    rec.flags |= dxv <= a.p.fb_tol ? CTM_BLK_VALID : CTM_BLK_FB_REJECT;
+    write_block(a, g.box, g.slot, rec);
+}
+
 }  // namespace ctm

@@ -187,11 +187,9 @@ MatchArgs make_args(const ctm_ctx *ctx, const ctm_frame *frames, const int32_t *
     a.nc_stride = ctx->nc_stride;
     a.strip_cols = ctx->strip_cols;
     a.strip_rows = ctx->strip_rows;
-    a.queue_rounds = ctx->queue_rounds;
     a.sm_count = ctx->sm_count;
     a.census_mode = ctx->census_mode;
     a.match_mode = ctx->match_mode;
-    a.split_ways = ctx->split_ways;
     if (!ctx->maps_ok) a.ws.tmaps = nullptr;
     a.stats_accumulate = 0;
     a.inject_expiry = 0;
@@ -202,8 +200,8 @@ MatchArgs make_args(const ctm_ctx *ctx, const ctm_frame *frames, const int32_t *
 // The launch sequence of one match call after the frame descriptors and counts
 // are in device memory: planning, census demand marking, census of the marked
 // tiles, matching.  direct: launched now, not captured into a graph (an armed
-// fault injection applies to such a launch of the fused persistent matcher
-// only, and is then disarmed).
+// fault injection applies to such a launch of the tensor-core matcher only, and
+// is then disarmed).
 int enqueue_match(ctm_ctx *ctx, const MatchArgs &a, int frames_grid, int match_grid, cudaStream_t s,
                   bool plain, int n_boxes_host, bool direct = true)
 {
@@ -220,7 +218,7 @@ int enqueue_match(ctm_ctx *ctx, const MatchArgs &a, int frames_grid, int match_g
     if (!plain) {
         if (e == cudaSuccess)
             e = ctx->match_mode == 1 ? launch_match_pipe(b, ctx->match_threads, match_grid, s)
-                                     : launch_match_persistent(b, ctx->match_threads, match_grid, s);
+                                     : launch_match_tc(b, s);
     } else {
         for (int i = 0; i < n_boxes_host && e == cudaSuccess; ++i)
             e = launch_match_box(b, ctx->match_threads, i, s);
@@ -356,14 +354,10 @@ int ctm_create(ctm_ctx **out, const ctm_params *p, int max_frames, int max_width
     const size_t o_base = take(sizeof(int) * (size_t)max_boxes);
     const size_t o_blocks = take(sizeof(int2) * (size_t)ctx->caps.max_blocks);
     const size_t o_blkres = take(sizeof(BlockResult) * (size_t)ctx->caps.max_blocks);
-    const size_t o_chunk = take(sizeof(ChunkState) * (size_t)ctx->caps.max_blocks);
     const size_t o_tmaps =
         take(max_frames <= kMaxMapFrames ? sizeof(CUtensorMap) * 4 * kBoxClasses * (size_t)max_frames : 0);
-    const size_t o_ccost = take(sizeof(int32_t) * (size_t)ctx->caps.max_blocks * ctx->nc_stride);
     const size_t o_geom = take(sizeof(BlockGeom) * (size_t)ctx->caps.max_blocks);
     const size_t o_queue = take(sizeof(int) * (size_t)ctx->caps.max_blocks);
-    const size_t o_queue_w = take(sizeof(int) * kQueueClasses * (size_t)ctx->caps.max_blocks);
-    const size_t o_sched = take(sizeof(int) * kSchedInts);
     const size_t o_counts = take(sizeof(Counts));
     const size_t o_stats = take(sizeof(Counts));
     const size_t o_frames = take(sizeof(ctm_frame) * (size_t)max_frames);
@@ -399,13 +393,9 @@ int ctm_create(ctm_ctx **out, const ctm_params *p, int max_frames, int max_width
     ws.blk_base = reinterpret_cast<int *>(base + o_base);
     ws.blocks = reinterpret_cast<int2 *>(base + o_blocks);
     ws.blkres = reinterpret_cast<BlockResult *>(base + o_blkres);
-    ws.chunk = reinterpret_cast<ChunkState *>(base + o_chunk);
     ws.tmaps = reinterpret_cast<const CUtensorMap *>(base + o_tmaps);
-    ws.chunk_cost = reinterpret_cast<int32_t *>(base + o_ccost);
     ws.geom = reinterpret_cast<BlockGeom *>(base + o_geom);
     ws.queue = reinterpret_cast<int *>(base + o_queue);
-    ws.queue_w = reinterpret_cast<int *>(base + o_queue_w);
-    ws.sched = reinterpret_cast<int *>(base + o_sched);
     ws.counts = reinterpret_cast<Counts *>(base + o_counts);
     ws.stats = reinterpret_cast<Counts *>(base + o_stats);
     ws.frames = reinterpret_cast<ctm_frame *>(base + o_frames);
@@ -422,7 +412,7 @@ int ctm_create(ctm_ctx **out, const ctm_params *p, int max_frames, int max_width
     }
     ctx->maps_ok = encode_plane_maps(ws, ctx->caps, k, const_cast<CUtensorMap *>(ws.tmaps));
     MatchArgs a = make_args(ctx, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
-    if (match_configure(a, ctx->match_threads, &ctx->ctas_per_sm) != cudaSuccess || ctx->ctas_per_sm < 1) {
+    if (match_configure(a, ctx->match_threads) != cudaSuccess || match_tc_configure() != cudaSuccess) {
         cudaGetLastError();
         ctm_destroy(ctx);
         return CTM_ECUDA;
@@ -601,8 +591,7 @@ int ctm_match_batch_profiled(ctm_ctx *ctx, const ctm_frame *frames_dev, const in
     if (e == cudaSuccess) e = launch_census_roi(a, ctx->sm_count, s);
     if (e == cudaSuccess) e = cudaEventRecord(ev[3], s);
     if (e == cudaSuccess)
-        e = ctx->match_mode == 1 ? launch_match_pipe(a, ctx->match_threads, grid, s)
-                                 : launch_match_persistent(a, ctx->match_threads, grid, s);
+        e = ctx->match_mode == 1 ? launch_match_pipe(a, ctx->match_threads, grid, s) : launch_match_tc(a, s);
     if (e == cudaSuccess) e = cudaEventRecord(ev[4], s);
     if (e == cudaSuccess) e = launch_aggregate(a, s);
     for (int i = 5; i < 8 && e == cudaSuccess; ++i) e = cudaEventRecord(ev[i], s);
@@ -901,9 +890,9 @@ int ctm_set_tuning(ctm_ctx *ctx, const ctm_tuning *t)
     trial.strip_cols = t->strip_cols;
     MatchArgs a = make_args(&trial, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
     int ctas = 0;
-    // the fused kernels stay configured either way (the per-box path uses them)
+    // the per-box kernels stay configured either way
     if (match_smem_bytes(a) > 227 * 1024) return CTM_EINVAL;
-    if (match_configure(a, t->match_threads, &ctas) != cudaSuccess || ctas < 1) {
+    if (match_configure(a, t->match_threads) != cudaSuccess) {
         cudaGetLastError();
         return CTM_EINVAL;
     }
@@ -968,19 +957,24 @@ int ctm_autotune(ctm_ctx *ctx, const ctm_frame *frames_dev, const int32_t *count
     ctm_tuning bt = cur;
     float bms = 3.4e38f;
     int status = CTM_OK;
-    // 1. matcher x CTA size x strip chunk width (joint), at the current census mode and split
-    // strip widths: the narrowest a point column fits (N_d + 2, rounded up to 8),
-    // then multiples of 32 above it
+    // 1. the tensor-core matcher (at the current CTA size and strip width, which it does
+    // not use), then the two-pass matcher: CTA size x strip chunk width -- the narrowest
+    // a point column fits (N_d + 2, rounded up to 8), then multiples of 32 above it
+    {
+        ctm_tuning t = bt;
+        t.match_mode = 0;
+        status = measure(t, &bms);
+        if (status == CTM_OK) bt = t;
+    }
     int widths[10];
     int nw = 0;
     widths[nw++] = (int)round_up(ctx->nd_max + 2, 8);
     for (int w = (int)round_up(ctx->nd_max + 2, 32); nw < 10; w += 32)
         if (w > widths[0]) widths[nw++] = w;
-    for (int mode = 0; mode <= 1 && status == CTM_OK; ++mode) {
-      for (int th = 128; th <= 256 && status == CTM_OK; th *= 2) {
+    for (int th = 128; th <= 256 && status == CTM_OK; th *= 2) {
         for (int wi = 0; wi < nw; ++wi) {
             ctm_tuning t = bt;
-            t.match_mode = mode;
+            t.match_mode = 1;
             t.match_threads = th;
             t.strip_cols = widths[wi];
             float ms = 0.0f;
@@ -989,30 +983,11 @@ int ctm_autotune(ctm_ctx *ctx, const ctm_frame *frames_dev, const int32_t *count
             if (r != CTM_OK) { status = r; break; }
             if (ms < bms) { bms = ms; bt = t; }
         }
-      }
     }
-    // 2. census variant, 3. per-SM rounds, one at a time around the best so far
-    const int modes[3] = {0, 1, 2};
-    for (int i = 0; i < 3 && status == CTM_OK; ++i) {
+    // 2. census variant
+    for (int m = 0; m < 3 && status == CTM_OK; ++m) {
         ctm_tuning t = bt;
-        t.census_mode = modes[i];
-        float ms = 0.0f;
-        const int r = measure(t, &ms);
-        if (r != CTM_OK) { status = r; break; }
-        if (ms < bms) { bms = ms; bt = t; }
-    }
-    for (int i = 0; i < 2 && status == CTM_OK; ++i) {
-        ctm_tuning t = bt;
-        t.queue_rounds = i;
-        float ms = 0.0f;
-        const int r = measure(t, &ms);
-        if (r != CTM_OK) { status = r; break; }
-        if (ms < bms) { bms = ms; bt = t; }
-    }
-    // 4. disparity-chunk tiles of the fused matcher: automatic or never
-    for (int sw = 0; sw <= 1 && status == CTM_OK && bt.match_mode == 0; ++sw) {
-        ctm_tuning t = bt;
-        t.split_ways = sw;
+        t.census_mode = m;
         float ms = 0.0f;
         const int r = measure(t, &ms);
         if (r != CTM_OK) { status = r; break; }

@@ -82,12 +82,17 @@ __device__ __forceinline__ bool mbar_wait_for(uint64_t *mbar, unsigned parity)
     return false;
 }
 
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *mbar, unsigned parity, int *error_flag)
+__device__ __noinline__ bool mbar_wait_slow(uint64_t *mbar, unsigned parity, int *error_flag)
 {
     if (mbar_wait_for(mbar, parity)) return true;
     atomicOr(error_flag, 1);
     mbar_wait_for(mbar, parity);
     return false;
+}
+
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *mbar, unsigned parity, int *error_flag)
+{
+    return mbar_try_wait(mbar, parity) || mbar_wait_slow(mbar, parity, error_flag);
 }
 
 struct Smem {

@@ -38,8 +38,6 @@ struct DeviceState {
     bool ready;
     unsigned char *base;  // device address of g_noalloc_scratch on this device
     int sm_count;
-    int match_need;       // matching kernel's shared-memory bytes last configured (0: none)
-    int match_ctas;       // its resident CTAs per SM at that size
 };
 DeviceState g_state[kMaxDevices];
 
@@ -60,6 +58,10 @@ int setup_device(int dev)
     }
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
+        cudaGetLastError();
+        return CTM_ECUDA;
+    }
+    if (ctm::match_tc_configure() != cudaSuccess) {
         cudaGetLastError();
         return CTM_ECUDA;
     }
@@ -157,13 +159,9 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     ws.blk_base = reinterpret_cast<int *>(b + o_base);
     ws.blocks = reinterpret_cast<int2 *>(b + o_blocks);
     ws.blkres = reinterpret_cast<BlockResult *>(b + o_blkres);
-    ws.chunk = nullptr;  // no disparity-chunk tiles: their state does not fit the array
     ws.tmaps = nullptr;  // strips load by 1-D bulk copies
-    ws.chunk_cost = nullptr;
     ws.geom = reinterpret_cast<BlockGeom *>(b + o_geom);
     ws.queue = reinterpret_cast<int *>(b + o_queue);
-    ws.queue_w = nullptr;  // one dynamic queue in sampling order (no per-SM rounds)
-    ws.sched = nullptr;
     ws.counts = reinterpret_cast<Counts *>(b + o_counts);
     ws.stats = reinterpret_cast<Counts *>(b + o_stats);
     ws.frames = reinterpret_cast<ctm_frame *>(b + o_frames);
@@ -190,26 +188,11 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     a.dbg.cost_b = nullptr;
     a.nc_stride = nd_max * ndy;
     a.strip_cols = strip_cols;
-    a.queue_rounds = 0;
     a.sm_count = ds.sm_count;
     a.census_mode = 0;
     a.match_mode = 0;
-    a.split_ways = 1;
     a.strip_rows = p->pts_side * ndy;
 
-    const int threads = 128;
-    DeviceState &dsm = g_state[dev];
-    const int need = (int)match_smem_bytes(a);
-    if (dsm.match_need != need) {  // attribute and occupancy queries only when the size changes
-        int ctas = 0;
-        if (match_configure_raise(a, threads, &ctas) != cudaSuccess || ctas < 1) {
-            cudaGetLastError();
-            return CTM_ECUDA;
-        }
-        dsm.match_need = need;
-        dsm.match_ctas = ctas;
-    }
-    const int ctas = dsm.match_ctas;
     census_roi_ctas_per_sm(p->win_w, p->win_h, 0);  // this window's occupancy query, cached after the first
     cudaStream_t s = (cudaStream_t)stream;
     // the census demand bitmap, the counters and the block counts must start at
@@ -222,9 +205,7 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     if (e == cudaSuccess) e = launch_plan(a, s);
     if (e == cudaSuccess) e = launch_sample(a, s);
     if (e == cudaSuccess) e = launch_census_roi(a, ds.sm_count, s);
-    const long long blocks_ub = (long long)std::max(n_boxes, 1) * std::max(p->grid_g * p->grid_g, 1);
-    const int grid = (int)std::min<long long>((long long)ds.sm_count * ctas, blocks_ub);
-    if (e == cudaSuccess) e = launch_match_persistent(a, threads, grid, s);
+    if (e == cudaSuccess) e = launch_match_tc(a, s);
     if (e == cudaSuccess) e = launch_aggregate(a, s);
     if (e != cudaSuccess) {
         cudaGetLastError();

@@ -274,8 +274,9 @@ __global__ void __launch_bounds__(256) sample_kernel(MatchArgs a)
     const BoxPlan P = a.ws.plans[box];
     const BlockRect r = block_rect(P, slot, a.p.pts_side);
     const int nx = r.nx, ny = r.ny;
-    const int Xl = lane < nx ? point_coord(r.bx0, r.bx1, nx, lane) : 0;
-    const int Yl = lane < ny ? point_coord(r.by0, r.by1, ny, lane) : 0;
+    // columns beyond nx and rows beyond ny repeat the last one (no point of theirs is usable)
+    const int Xl = nx > 0 ? point_coord(r.bx0, r.bx1, nx, min(lane, nx - 1)) : 0;
+    const int Yl = ny > 0 ? point_coord(r.by0, r.by1, ny, min(lane, ny - 1)) : 0;
     int4 occ = make_int4(0, 0, 0, 0);
     if (lane < P.nocc) occ = a.ws.occ[(long long)box * kMaxOcc + lane];
     // usable: left census defined (window inside the grid) and full-res position
@@ -358,11 +359,6 @@ __global__ void __launch_bounds__(256) sample_kernel(MatchArgs a)
         }
     } else {
         if (lane == 0) {
-            if (a.ws.chunk) {  // state for disparity-chunk tiles (used only when the queue is short)
-                ChunkState cs{};
-                cs.fkey = cs.bkey = 0xffffffffu;
-                a.ws.chunk[b] = cs;
-            }
             const int work = n_valid * nd * ndy;
             if (work >= kBigWork) {
                 const int q = atomicAdd(&a.ws.counts->n_big, 1);
@@ -370,11 +366,6 @@ __global__ void __launch_bounds__(256) sample_kernel(MatchArgs a)
             } else {
                 const int q = atomicAdd(&a.ws.counts->n_small, 1);
                 a.ws.queue[a.caps.max_blocks - 1 - q] = b;
-            }
-            if (work_queue_on(a, a.ws.counts->n_blocks)) {
-                const int c = queue_class(work);
-                const int q = atomicAdd(&a.ws.counts->n_class[c], 1);
-                a.ws.queue_w[(long long)c * a.caps.max_blocks + q] = b;
             }
         }
         // census demand of the searchable block (see mark_range)
@@ -420,15 +411,12 @@ cudaError_t launch_sample(const MatchArgs &a, cudaStream_t s)
 // It is the last kernel of a call, so it also leaves the workspace ready for
 // the next one: block 0 moves the counters to the stats record and zeroes
 // them -- all but the error flag, which every CTA reads here and the next
-// call's plan_kernel clears -- and the matcher's round counters, and every
-// box's block count goes back to zero (no memset nodes at the start of a call).
+// call's plan_kernel clears -- and every box's block count goes back to zero (no memset nodes at the start of a call).
 __global__ void __launch_bounds__(256) aggregate_kernel(MatchArgs a)
 {
     __shared__ float scratch[8][2 * kMaxSlots];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int failed = *reinterpret_cast<volatile int *>(&a.ws.counts->error);
-    if (blockIdx.x == 0 && a.ws.sched)
-        for (int i = threadIdx.x; i < kSchedInts; i += blockDim.x) a.ws.sched[i] = 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const Counts c = *a.ws.counts;
         if (a.stats_accumulate) {  // a later sub-batch of one call
@@ -443,7 +431,6 @@ __global__ void __launch_bounds__(256) aggregate_kernel(MatchArgs a)
             t.n_small += c.n_small;
             t.n_tiles += c.n_tiles;
             t.host_bytes += c.host_bytes;
-            for (int i = 0; i < kQueueClasses; ++i) t.n_class[i] += c.n_class[i];
             *a.ws.stats = t;
         } else {
             *a.ws.stats = c;
