@@ -352,7 +352,6 @@ int ctm_create(ctm_ctx **out, const ctm_params *p, int max_frames, int max_width
     const size_t o_occ = take(sizeof(int4) * (size_t)max_boxes * kMaxOcc);
     const size_t o_nblk = take(sizeof(int) * (size_t)max_boxes);
     const size_t o_base = take(sizeof(int) * (size_t)max_boxes);
-    const size_t o_blocks = take(sizeof(int2) * (size_t)ctx->caps.max_blocks);
     const size_t o_blkres = take(sizeof(BlockResult) * (size_t)ctx->caps.max_blocks);
     const size_t o_tmaps =
         take(max_frames <= kMaxMapFrames ? sizeof(CUtensorMap) * 4 * kBoxClasses * (size_t)max_frames : 0);
@@ -391,7 +390,6 @@ int ctm_create(ctm_ctx **out, const ctm_params *p, int max_frames, int max_width
     ws.occ = reinterpret_cast<int4 *>(base + o_occ);
     ws.nblk = reinterpret_cast<int *>(base + o_nblk);
     ws.blk_base = reinterpret_cast<int *>(base + o_base);
-    ws.blocks = reinterpret_cast<int2 *>(base + o_blocks);
     ws.blkres = reinterpret_cast<BlockResult *>(base + o_blkres);
     ws.tmaps = reinterpret_cast<const CUtensorMap *>(base + o_tmaps);
     ws.geom = reinterpret_cast<BlockGeom *>(base + o_geom);

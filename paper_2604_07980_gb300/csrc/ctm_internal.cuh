@@ -96,8 +96,7 @@ struct Workspace {
     int4 *occ;                 // [max_boxes * kMaxOcc]
     int *nblk;                 // [max_boxes]
     int *blk_base;             // [max_boxes]
-    int2 *blocks;              // [max_blocks] (box, slot), flat in box order
-    BlockGeom *geom;           // [max_blocks] indexed like blocks
+    BlockGeom *geom;           // [max_blocks] blk_base[box] + slot
     int *queue;                // [max_blocks] searchable blocks: large from the front, small from the back
     BlockResult *blkres;       // [max_blocks]
     const CUtensorMap *tmaps;  // [max_frames * 4 * kBoxClasses] census planes L1, R1, Lk, Rk as 2-D
@@ -156,31 +155,22 @@ __device__ __forceinline__ int queue_at(const MatchArgs &a, int n_big, int p)
     return p < n_big ? a.ws.queue[p] : a.ws.queue[a.caps.max_blocks - 1 - (p - n_big)];
 }
 
+// num / den for 0 <= num < 2^24 and 1 <= den < 2^24: one approximate fp32 quotient (off by
+// less than one) and a correction, a third of the instructions of an integer division.
+__device__ __forceinline__ int div_small(int num, int den)
+{
+    int q = (int)__fdividef((float)num, (float)den);
+    const int r = num - q * den;
+    q += r >= den ? 1 : 0;
+    q -= r < 0 ? 1 : 0;
+    return q;
+}
+
 // Sampled coordinate j of n on [b0, b1): the centre of the j-th of n equal cells
 // (Sec. 4.3.4's regular point grid).
 __device__ __forceinline__ int point_coord(int b0, int b1, int n, int j)
 {
-    return b0 + ((2 * j + 1) * (b1 - b0)) / (2 * n);
-}
-
-// Rectangle of block `slot` (row-major in a g x g grid) of a planned box, on its
-// matching grid, and its point counts per side.
-struct BlockRect {
-    int bx0, by0, bx1, by1, nx, ny;
-};
-
-__device__ __forceinline__ BlockRect block_rect(const BoxPlan &P, int slot, int pts_side)
-{
-    BlockRect r;
-    const int ga = slot % P.g, gb = slot / P.g;
-    const int bw = P.sx1 - P.sx0, bh = P.sy1 - P.sy0;
-    r.bx0 = P.sx0 + (ga * bw) / P.g;
-    r.bx1 = P.sx0 + ((ga + 1) * bw) / P.g;
-    r.by0 = P.sy0 + (gb * bh) / P.g;
-    r.by1 = P.sy0 + ((gb + 1) * bh) / P.g;
-    r.nx = min(r.bx1 - r.bx0, pts_side);
-    r.ny = min(r.by1 - r.by0, pts_side);
-    return r;
+    return b0 + div_small((2 * j + 1) * (b1 - b0), 2 * n);
 }
 
 // Census launches (census.cu)

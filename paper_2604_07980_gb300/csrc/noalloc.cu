@@ -133,7 +133,6 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     const size_t o_occ = take(sizeof(int4) * (size_t)kMaxBoxes * kMaxOcc);
     const size_t o_nblk = take(sizeof(int) * kMaxBoxes);
     const size_t o_base = take(sizeof(int) * kMaxBoxes);
-    const size_t o_blocks = take(sizeof(int2) * (size_t)caps.max_blocks);
     const size_t o_blkres = take(sizeof(BlockResult) * (size_t)caps.max_blocks);
     const size_t o_geom = take(sizeof(BlockGeom) * (size_t)caps.max_blocks);
     const size_t o_queue = take(sizeof(int) * (size_t)caps.max_blocks);
@@ -157,7 +156,6 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     ws.occ = reinterpret_cast<int4 *>(b + o_occ);
     ws.nblk = reinterpret_cast<int *>(b + o_nblk);
     ws.blk_base = reinterpret_cast<int *>(b + o_base);
-    ws.blocks = reinterpret_cast<int2 *>(b + o_blocks);
     ws.blkres = reinterpret_cast<BlockResult *>(b + o_blkres);
     ws.tmaps = nullptr;  // strips load by 1-D bulk copies
     ws.geom = reinterpret_cast<BlockGeom *>(b + o_geom);

@@ -7,10 +7,10 @@
 // blocks, and select its occluders -- overlapping boxes of the same frame with a
 // larger bottom y (Sec. 4.3.5), nearest (largest bottom y) first, at most
 // max_occluders.  Boxes that are empty after clipping get their outputs here.
-// Each slice's blocks get a contiguous range of the flat (box, slot) block list.
+// Each slice's blocks get a contiguous range of block indices.
 //
-// sample_kernel (one warp per block): the block's point grid and its usable
-// points; blocks with fewer than min_pts usable points are finished here, the
+// sample_kernel (one warp per row of a box's block grid): the blocks' point grids and
+// usable points; blocks with fewer than min_pts usable points are finished here, the
 // others go to the work queue (large work first) and mark the census tiles
 // their search can read.  All counts come from device memory so a captured
 // graph replays with new inputs.
@@ -70,7 +70,7 @@ constexpr int kKeyCache = 8;       // occluder keys per lane held in registers
 // map to the matching grid and select the occluders of every box of the slice
 // (the frame's clipped boxes are staged in shared memory for the pairwise
 // test), then the slice's block counts are scanned and one atomic reserves the
-// slice's range of the flat block list.
+// slice's range of block indices.
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(MatchArgs a, int S)
 {
     __shared__ int4 sbox[kStageBoxes];
@@ -231,21 +231,10 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(MatchArgs a, int S)
     if (tid == 0) s_base = atomicAdd(&a.ws.counts->n_blocks, s_run);
     __syncthreads();
     const int base = s_base;
-    // a warp per box writes the box's entries of the flat block list
-    for (int i = sb + warp; i < se; i += kPlanThreads / 32) {
-        const int bb = base + a.ws.blk_base[i];
-        const int v = a.ws.nblk[i];
-        __syncwarp();
-        if (lane == 0) a.ws.blk_base[i] = bb;
-        for (int s2 = lane; s2 < v; s2 += 32) a.ws.blocks[bb + s2] = make_int2(i, s2);
-    }
+    for (int i = sb + tid; i < se; i += blockDim.x) a.ws.blk_base[i] += base;
 }
 
-// Mark, for one block, the census row tiles its two passes can read: the left
-// plane at the sampled rows (plus the vertical spread of the backward pass) over
-// [X_0 - (dmax - dmin), X_last + (dmax - dmin)], which holds the points and every
-// backward strip; the right plane at rows Y_m + dy over [X_0 - dmax, X_last - dmin],
-// which holds every forward strip and the backward queries.
+// Mark the census row tiles of plane q that columns [c0, c1] of row y lie in.
 __device__ __forceinline__ void mark_range(const MatchArgs &a, int f, int q, int y, int c0, int c1,
                                            int Ws, int Hs)
 {
@@ -263,139 +252,184 @@ __device__ __forceinline__ void mark_range(const MatchArgs &a, int f, int q, int
     }
 }
 
-__global__ void __launch_bounds__(256) sample_kernel(MatchArgs a)
+// Mark what the searches of neighbouring blocks of one grid row can read, whose sampled
+// columns span [x_first, x_last]: the left plane at the sampled rows (lane m holds row
+// m; plus the vertical spread of the backward pass) over [x_first - (dmax - dmin),
+// x_last + (dmax - dmin)], which holds the points and every backward strip; the right
+// plane at rows Y_m + dy over [x_first - dmax, x_last - dmin], which holds every forward
+// strip and the backward queries.
+__device__ __forceinline__ void mark_blocks(const MatchArgs &a, const BoxPlan &P, int ny, int Yl, int x_first,
+                                            int x_last)
+{
+    const int lane = threadIdx.x & 31;
+    const int qL = (P.far || a.p.close_factor == 1) ? 0 : 2;
+    const int span = P.dmax - P.dmin;
+    const int dyr = a.p.dy_max - a.p.dy_min;
+    const int nl = 2 * dyr + 1, nr = dyr + 1;
+    const int items = ny * (nl + nr);
+    for (int it0 = 0; it0 < items; it0 += 32) {  // uniform trip count: the shuffle needs every lane
+        const int it = it0 + lane;
+        const int m = dyr == 0 ? (it >> 1) & 15 : (it < items ? it : 0) / (nl + nr);
+        const int e = it - m * (nl + nr);
+        const int y = __shfl_sync(0xffffffffu, Yl, m);
+        if (it >= items) continue;
+        if (e < nl)
+            mark_range(a, P.frame, qL, y + e - dyr, x_first - span, x_last + span, P.Ws, P.Hs);
+        else
+            mark_range(a, P.frame, qL + 1, y + a.p.dy_min + (e - nl), x_first - P.dmax, x_last - P.dmin, P.Ws,
+                       P.Hs);
+    }
+}
+
+// One warp per row of a box's block grid (FAR boxes: one row of one block), a half-warp
+// per block.  The row's blocks share the sampled rows, their occluded rows and mostly
+// their census tiles.  Bound by its instructions (the point grids' divisions, the
+// occluders, the records) and the census marks' atomics, of which neighbouring blocks
+// with touching ranges make one set.  A warp per block took 24.5 us on 32 frames of
+// 1920x1200 (18 K blocks) and 36.9 us on 8 of 3840x2160 (38 K); this 15.1 and 22.3 us.
+__global__ void __launch_bounds__(256) sample_kernel(MatchArgs a, int rows_per_box)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int b = blockIdx.x * 8 + warp;
-    if (b >= a.ws.counts->n_blocks) return;
-    const int2 bs = a.ws.blocks[b];
-    const int box = bs.x, slot = bs.y;
+    const int wi = blockIdx.x * 8 + warp;
+    const int box = wi / rows_per_box, gb = wi - box * rows_per_box;
+    if (box >= a.ws.counts->n_boxes || a.ws.nblk[box] == 0) return;
     const BoxPlan P = a.ws.plans[box];
-    const BlockRect r = block_rect(P, slot, a.p.pts_side);
-    const int nx = r.nx, ny = r.ny;
-    // columns beyond nx and rows beyond ny repeat the last one (no point of theirs is usable)
-    const int Xl = nx > 0 ? point_coord(r.bx0, r.bx1, nx, min(lane, nx - 1)) : 0;
-    const int Yl = ny > 0 ? point_coord(r.by0, r.by1, ny, min(lane, ny - 1)) : 0;
+    if (gb >= P.g) return;
+    const int base = a.ws.blk_base[box] + gb * P.g;
+    // the sampled rows; rows beyond ny repeat the last one (no point of theirs is usable)
+    const int bw = P.sx1 - P.sx0, bh = P.sy1 - P.sy0;
+    const int by0 = P.sy0 + div_small(gb * bh, P.g), by1 = P.sy0 + div_small((gb + 1) * bh, P.g);
+    const int ny = min(by1 - by0, a.p.pts_side);
+    const int Yl = ny > 0 ? point_coord(by0, by1, ny, min(lane, ny - 1)) : 0;
+    // usable: left census defined (window inside the grid) and full-res position
+    // k (x, y) in no kept occluder.  Each occluder covers a column range x a row range of
+    // the point grid: lane q holds occluder q and the rows it covers.
+    const int sxw = a.p.win_w >> 1, syw = a.p.win_h >> 1;
+    const unsigned rowok = __ballot_sync(full, lane < ny && Yl - syw >= 0 && Yl + syw < P.Hs);
     int4 occ = make_int4(0, 0, 0, 0);
     if (lane < P.nocc) occ = a.ws.occ[(long long)box * kMaxOcc + lane];
-    // usable: left census defined (window inside the grid) and full-res position
-    // k (x, y) in no kept occluder
-    const int sxw = a.p.win_w >> 1, syw = a.p.win_h >> 1;
-    const bool col_ok = lane < nx && Xl - sxw >= 0 && Xl + sxw < P.Ws;
-    // Each occluder covers a column range x a row range of the point grid: lane q
-    // forms the row mask of occluder q, then every column lane removes the rows
-    // of the occluders whose x range holds it.
-    const unsigned rowok = __ballot_sync(full, lane < ny && Yl - syw >= 0 && Yl + syw < P.Hs);
     unsigned occrows = 0u;
-    if (P.nocc > 0) {
-        for (int m = 0; m < ny; ++m) {
-            const int fy = P.k * __shfl_sync(full, Yl, m);
-            if (lane < P.nocc && fy >= occ.y && fy < occ.w) occrows |= 1u << m;
-        }
-    }
-    unsigned colmask = col_ok ? rowok : 0u;
-    const int fx = P.k * Xl;
+    const int fy = lane < ny ? P.k * Yl : -1;
     for (int q = 0; q < P.nocc; ++q) {
-        const int ox0 = __shfl_sync(full, occ.x, q), ox1 = __shfl_sync(full, occ.z, q);
-        const unsigned rows = __shfl_sync(full, occrows, q);
-        if (fx >= ox0 && fx < ox1) colmask &= ~rows;
+        const int oy0 = __shfl_sync(full, occ.y, q), oy1 = __shfl_sync(full, occ.w, q);
+        const unsigned rows = __ballot_sync(full, fy >= oy0 && fy < oy1);
+        if (lane == q) occrows = rows;
     }
-    const int cnt = __popc(colmask);
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(full, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const int n_valid = __shfl_sync(full, incl, 31);
-    // column chunks whose strip (plus alignment) fits the shared-memory strip
+    const unsigned live = __ballot_sync(full, occrows != 0u);  // occluders that touch these rows
     const int nd = P.dmax - P.dmin + 1;
-    unsigned cstart = 1u;
-    {
-        int x0 = __shfl_sync(full, Xl, 0);
-        for (int j = 1; j < nx; ++j) {
-            const int xj = __shfl_sync(full, Xl, j);
-            if (xj - x0 + nd + 2 > a.strip_cols) {
-                cstart |= 1u << j;
-                x0 = xj;
-            }
-        }
-    }
-    BlockGeom *g = a.ws.geom + b;
-    if (lane < kMaxPtsSide) {
-        g->X[lane] = (int16_t)Xl;
-        g->Y[lane] = (int16_t)Yl;
-        g->colmask[lane] = (uint16_t)colmask;
-        g->colprefix[lane] = (uint16_t)(incl - cnt);
-    }
-    if (lane == 0) {
-        g->n_valid = n_valid;
-        g->nx = nx;
-        g->ny = ny;
-        g->cstart = cstart;
-        g->box = box;
-        g->slot = slot;
-        g->frame = P.frame;
-        g->k = P.k;
-        g->far = P.far;
-        g->dmin = P.dmin;
-        g->dmax = P.dmax;
-        g->Ws = P.Ws;
-        g->Hs = P.Hs;
-    }
     const int ndy = a.p.dy_max - a.p.dy_min + 1;
-    if (n_valid < a.p.min_pts) {
-        if (lane == 0) {
-            ctm_block rec;
-            rec.n_pts = nx * ny;
-            rec.n_valid = n_valid;
-            rec.d_f = rec.dy_f = rec.d_b = rec.dy_b = 0;
-            rec.s_m = rec.s_0 = rec.s_p = 0;
-            rec.d_sub = 0.0f;
-            rec.d_full = 0.0f;
-            rec.flags = CTM_BLK_PRESENT | CTM_BLK_FEW_POINTS;
-            write_block(a, box, slot, rec);
+    int work = 0;  // lane ga: usable points x candidates of a searchable block, else 0
+    int m0 = 1, m1 = 0;  // columns of the blocks not marked yet (none)
+    const int half = lane >> 4, hl = lane & 15;
+    const int Yh = __shfl_sync(full, Yl, hl);
+    for (int ga0 = 0; ga0 < P.g; ga0 += 2) {
+        const int ga = ga0 + half;  // this half-warp's block, its lanes the block's columns
+        const bool on = ga < P.g;
+        const int bx0 = P.sx0 + div_small(ga * bw, P.g), bx1 = P.sx0 + div_small((ga + 1) * bw, P.g);
+        const int nx = on ? min(bx1 - bx0, a.p.pts_side) : 0;
+        const int Xl = nx > 0 ? point_coord(bx0, bx1, nx, min(hl, nx - 1)) : 0;
+        unsigned colmask = hl < nx && Xl - sxw >= 0 && Xl + sxw < P.Ws ? rowok : 0u;
+        const int fx = P.k * Xl;
+        for (unsigned o = live; o; o &= o - 1u) {
+            const int q = __ffs(o) - 1;
+            const int ox0 = __shfl_sync(full, occ.x, q), ox1 = __shfl_sync(full, occ.z, q);
+            const unsigned rows = __shfl_sync(full, occrows, q);
+            if (fx >= ox0 && fx < ox1) colmask &= ~rows;
         }
-    } else {
-        if (lane == 0) {
-            const int work = n_valid * nd * ndy;
-            if (work >= kBigWork) {
-                const int q = atomicAdd(&a.ws.counts->n_big, 1);
-                a.ws.queue[q] = b;
-            } else {
-                const int q = atomicAdd(&a.ws.counts->n_small, 1);
-                a.ws.queue[a.caps.max_blocks - 1 - q] = b;
+        const int cnt = __popc(colmask);
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < kMaxPtsSide; o <<= 1) {
+            const int y = __shfl_up_sync(full, incl, o, kMaxPtsSide);
+            if (hl >= o) incl += y;
+        }
+        const int n_valid = __shfl_sync(full, incl, 15, kMaxPtsSide);
+        const int x_first = __shfl_sync(full, Xl, 0, kMaxPtsSide), x_last = __shfl_sync(full, Xl, 15, kMaxPtsSide);
+        // column chunks whose strip (plus alignment) fits the popcount matchers' strip
+        unsigned cstart = 1u;
+        if (__any_sync(full, x_last - x_first + nd + 2 > a.strip_cols)) {
+            int x0 = x_first;
+            for (int j = 1; j < kMaxPtsSide; ++j) {
+                const int xj = __shfl_sync(full, Xl, j, kMaxPtsSide);
+                if (j < nx && xj - x0 + nd + 2 > a.strip_cols) {
+                    cstart |= 1u << j;
+                    x0 = xj;
+                }
             }
         }
-        // census demand of the searchable block (see mark_range)
-        const int x_first = __shfl_sync(full, Xl, 0), x_last = __shfl_sync(full, Xl, nx - 1);
-        const int qL = (P.far || a.p.close_factor == 1) ? 0 : 2;
-        const int span = P.dmax - P.dmin;
-        const int dyr = a.p.dy_max - a.p.dy_min;
-        const int nl = 2 * dyr + 1, nr = dyr + 1;
-        const int items = ny * (nl + nr);
-        for (int it0 = 0; it0 < items; it0 += 32) {  // uniform trip count: the shuffle needs every lane
-            const int it = it0 + lane;
-            const int m = (it < items ? it : 0) / (nl + nr);
-            const int e = it - m * (nl + nr);
-            const int y = __shfl_sync(full, Yl, m);
-            if (it >= items) continue;
-            if (e < nl)
-                mark_range(a, P.frame, qL, y + e - dyr, x_first - span, x_last + span, P.Ws, P.Hs);
-            else
-                mark_range(a, P.frame, qL + 1, y + a.p.dy_min + (e - nl), x_first - P.dmax, x_last - P.dmin,
-                           P.Ws, P.Hs);
+        const bool few = n_valid < a.p.min_pts;
+        if (on) {
+            BlockGeom *g = a.ws.geom + (base + ga);
+            g->X[hl] = (int16_t)Xl;
+            g->Y[hl] = (int16_t)Yh;
+            g->colmask[hl] = (uint16_t)colmask;
+            g->colprefix[hl] = (uint16_t)(incl - cnt);
+            if (hl == 0) {
+                g->n_valid = n_valid;
+                g->nx = nx;
+                g->ny = ny;
+                g->cstart = cstart;
+                g->box = box;
+                g->slot = gb * P.g + ga;
+                g->frame = P.frame;
+                g->k = P.k;
+                g->far = P.far;
+                g->dmin = P.dmin;
+                g->dmax = P.dmax;
+                g->Ws = P.Ws;
+                g->Hs = P.Hs;
+                if (few) {
+                    ctm_block rec;
+                    rec.n_pts = nx * ny;
+                    rec.n_valid = n_valid;
+                    rec.d_f = rec.dy_f = rec.d_b = rec.dy_b = 0;
+                    rec.s_m = rec.s_0 = rec.s_p = 0;
+                    rec.d_sub = 0.0f;
+                    rec.d_full = 0.0f;
+                    rec.flags = CTM_BLK_PRESENT | CTM_BLK_FEW_POINTS;
+                    write_block(a, box, gb * P.g + ga, rec);
+                }
+            }
+        }
+        const unsigned found = __ballot_sync(full, on && !few);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (!((found >> (16 * h)) & 1u)) continue;
+            const int nv = __shfl_sync(full, n_valid, 16 * h);
+            if (lane == ga0 + h) work = nv * nd * ndy;
+            // census demand: joined with the searchable block before it where the ranges touch
+            const int xf = __shfl_sync(full, x_first, 16 * h), xl = __shfl_sync(full, x_last, 16 * h);
+            if (m0 <= m1 && xf - m1 > nd) {
+                mark_blocks(a, P, ny, Yl, m0, m1);
+                m0 = 1;
+                m1 = 0;
+            }
+            if (m0 > m1) m0 = xf;
+            m1 = xl;
         }
     }
+    if (m0 <= m1) mark_blocks(a, P, ny, Yl, m0, m1);
+    // queue the searchable blocks, one reservation per end for the whole row
+    const unsigned big = __ballot_sync(full, work >= kBigWork), small = __ballot_sync(full, work > 0 && work < kBigWork);
+    int qb = 0, qs = 0;
+    if (lane == 0 && big) qb = atomicAdd(&a.ws.counts->n_big, __popc(big));
+    if (lane == 0 && small) qs = atomicAdd(&a.ws.counts->n_small, __popc(small));
+    qb = __shfl_sync(full, qb, 0);
+    qs = __shfl_sync(full, qs, 0);
+    const unsigned lt = (1u << lane) - 1u;
+    if (work >= kBigWork)
+        a.ws.queue[qb + __popc(big & lt)] = base + lane;
+    else if (work > 0)
+        a.ws.queue[a.caps.max_blocks - 1 - qs - __popc(small & lt)] = base + lane;
 }
 
 }  // namespace
 
 cudaError_t launch_sample(const MatchArgs &a, cudaStream_t s)
 {
-    const int grid = ceil_div_nn(a.caps.max_blocks, 8);
-    sample_kernel<<<grid, 256, 0, s>>>(a);
+    const int rows = std::max(a.p.grid_g, 1);
+    sample_kernel<<<ceil_div_nn(a.caps.max_boxes * rows, 8), 256, 0, s>>>(a, rows);
     return cudaGetLastError();
 }
 
