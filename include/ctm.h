@@ -208,7 +208,9 @@ int ctm_census_build(const uint8_t *img_dev, int width, int height, int pitch, i
  * (uint8 CTM_BOX_*).  dbg may be NULL.  The launch sequence of the batch path on
  * one frame: device planning and point sampling, the census of the row tiles the
  * search reads (both images, both resolutions), one persistent matching kernel
- * and a per-box aggregation kernel.  Errors: CTM_EINVAL, CTM_ENOMEM (beyond
+ * and a per-box aggregation kernel.  From a context's second call on the launches
+ * replay as a CUDA graph of the context, whose arguments each call sets (not with dbg,
+ * nor while `stream` is being captured).  Errors: CTM_EINVAL, CTM_ENOMEM (beyond
  * capacity), CTM_ECUDA. */
 int ctm_match_boxes(ctm_ctx *ctx, const uint8_t *left_dev, const uint8_t *right_dev,
                     int width, int height, int pitch, const ctm_box *boxes_dev, int n_boxes,

@@ -639,8 +639,7 @@ __global__ void __launch_bounds__(256) tile_list_kernel(MatchArgs a)
 {
     __shared__ int warp_tot[8];
     __shared__ int s_base;
-    int nf = a.counts_in[0];
-    nf = nf < 0 ? 0 : (nf > a.caps.max_frames ? a.caps.max_frames : nf);
+    const int nf = a.ws.counts->n_frames;  // clamped by the planner
     const long long total = (long long)nf * a.ws.bm_frame_words;
     const long long w0 = (long long)blockIdx.x * blockDim.x;
     if (w0 >= total) return;  // uniform per CTA

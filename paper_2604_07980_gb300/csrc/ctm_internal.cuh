@@ -104,8 +104,6 @@ struct Workspace {
                                // loads by tile::gather4); null: 1-D bulk copies, one per row
     Counts *counts;            // counters of the call in progress (zero between calls)
     Counts *stats;             // the last finished call's counters
-    ctm_frame *frames;         // staging for single-frame calls [max_frames]
-    int *counts_in;            // staging {n_frames, n_boxes}
     // census demand bitmap: one bit per kCensusTilePx-pixel tile of a plane row, per frame
     // planes in the order L1, R1, Lk, Rk; words = 32 tiles
     uint32_t *bitmap;
@@ -125,8 +123,10 @@ struct MatchArgs {
     Workspace ws;
     Caps caps;
     ctm_params p;
-    const ctm_frame *frames;   // device
-    const int *counts_in;      // device {n_frames, n_boxes}
+    const ctm_frame *frames;   // device; null: the one frame frame1 with n_boxes1 boxes
+    const int *counts_in;      // device {n_frames, n_boxes} (with frames)
+    ctm_frame frame1;          // single-frame calls
+    int n_boxes1;
     const ctm_box *boxes;      // device
     float *disp;
     float *depth;
@@ -202,7 +202,6 @@ cudaError_t launch_census_roi(const MatchArgs &a, int sm_count, cudaStream_t s);
 size_t census_smem_bytes(int win_h);
 
 // Planning (plan.cu)
-cudaError_t launch_stage_frame(const MatchArgs &a, ctm_frame f, int n_boxes, cudaStream_t s);
 cudaError_t launch_plan(const MatchArgs &a, cudaStream_t s);
 cudaError_t launch_aggregate(const MatchArgs &a, cudaStream_t s);
 cudaError_t launch_sample(const MatchArgs &a, cudaStream_t s);

@@ -136,8 +136,6 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     const size_t o_blkres = take(sizeof(BlockResult) * (size_t)caps.max_blocks);
     const size_t o_geom = take(sizeof(BlockGeom) * (size_t)caps.max_blocks);
     const size_t o_queue = take(sizeof(int) * (size_t)caps.max_blocks);
-    const size_t o_frames = take(sizeof(ctm_frame));
-    const size_t o_cin = take(sizeof(int) * 4);
     const size_t o_bm = take(sizeof(uint32_t) * (size_t)plane_off[4]);
     const size_t o_tiles = take(sizeof(unsigned long long) * 32 * (size_t)plane_off[4]);
     const size_t o_planes = take(sizeof(PlaneDesc) * 4);
@@ -162,8 +160,6 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     ws.queue = reinterpret_cast<int *>(b + o_queue);
     ws.counts = reinterpret_cast<Counts *>(b + o_counts);
     ws.stats = reinterpret_cast<Counts *>(b + o_stats);
-    ws.frames = reinterpret_cast<ctm_frame *>(b + o_frames);
-    ws.counts_in = reinterpret_cast<int *>(b + o_cin);
     ws.bitmap = reinterpret_cast<uint32_t *>(b + o_bm);
     ws.tiles = reinterpret_cast<unsigned long long *>(b + o_tiles);
     ws.planes = reinterpret_cast<PlaneDesc *>(b + o_planes);
@@ -175,8 +171,10 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     a.stats_accumulate = 0;
     a.inject_expiry = 0;
     a.gather_src = nullptr;
-    a.frames = ws.frames;
-    a.counts_in = ws.counts_in;
+    a.frames = nullptr;
+    a.counts_in = nullptr;
+    a.frame1 = ctm_frame{left_dev, right_dev, width, height, pitch, 0, n_boxes, f_px, baseline_m};
+    a.n_boxes1 = n_boxes;
     a.boxes = boxes_dev;
     a.disp = disp_dev;
     a.depth = depth_dev;
@@ -198,8 +196,6 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     cudaError_t e = cudaMemsetAsync(ws.bitmap, 0, sizeof(uint32_t) * (size_t)plane_off[4], s);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.counts, 0, sizeof(Counts), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.nblk, 0, sizeof(int) * kMaxBoxes, s);
-    const ctm_frame fr{left_dev, right_dev, width, height, pitch, 0, n_boxes, f_px, baseline_m};
-    if (e == cudaSuccess) e = launch_stage_frame(a, fr, n_boxes, s);
     if (e == cudaSuccess) e = launch_plan(a, s);
     if (e == cudaSuccess) e = launch_sample(a, s);
     if (e == cudaSuccess) e = launch_census_roi(a, ds.sm_count, s);

@@ -56,13 +56,6 @@ __device__ __forceinline__ bool overlaps(int4 a, int4 b)
     return ix1 > ix0 && iy1 > iy0;
 }
 
-__global__ void stage_frame_kernel(ctm_frame *frames, int *counts_in, ctm_frame f, int n_boxes)
-{
-    frames[0] = f;
-    counts_in[0] = 1;
-    counts_in[1] = n_boxes;
-}
-
 constexpr int kStageBoxes = 1024;  // boxes of one frame staged in shared memory
 constexpr int kKeyCache = 8;       // occluder keys per lane held in registers
 
@@ -77,8 +70,8 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(MatchArgs a, int S)
     __shared__ int warp_tot[kPlanThreads / 32];
     __shared__ int s_run, s_base;
     const int f = blockIdx.x / S, slice = blockIdx.x % S;
-    const int nf = clampi(a.counts_in[0], 0, a.caps.max_frames);
-    const int nb_total = clampi(a.counts_in[1], 0, a.caps.max_boxes);
+    const int nf = a.frames ? clampi(a.counts_in[0], 0, a.caps.max_frames) : 1;
+    const int nb_total = clampi(a.frames ? a.counts_in[1] : a.n_boxes1, 0, a.caps.max_boxes);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (blockIdx.x == 0 && tid == 0) {
         a.ws.counts->n_frames = nf;
@@ -86,7 +79,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(MatchArgs a, int S)
         a.ws.counts->error = 0;  // the previous call's flag stays until here (see aggregate_kernel)
     }
     if (f >= nf) return;
-    const ctm_frame fr = a.frames[f];
+    const ctm_frame fr = a.frames ? a.frames[f] : a.frame1;
     const bool bad_frame = fr.width < 1 || fr.height < 1 || fr.width > a.caps.max_width ||
                            fr.height > a.caps.max_height || fr.pitch < fr.width ||
                            fr.left == nullptr || fr.right == nullptr;
@@ -474,7 +467,7 @@ __global__ void __launch_bounds__(256) aggregate_kernel(MatchArgs a)
         *a.ws.counts = z;
     }
     const int box = blockIdx.x * 8 + warp;
-    if (box >= clampi(a.counts_in[1], 0, a.caps.max_boxes)) return;
+    if (box >= clampi(a.frames ? a.counts_in[1] : a.n_boxes1, 0, a.caps.max_boxes)) return;
     if (a.ws.nblk[box] == 0) return;
     if (failed) {
         if (lane == 0) {
@@ -492,12 +485,6 @@ __global__ void __launch_bounds__(256) aggregate_kernel(MatchArgs a)
 cudaError_t launch_aggregate(const MatchArgs &a, cudaStream_t s)
 {
     aggregate_kernel<<<ceil_div_nn(a.caps.max_boxes, 8), 256, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_stage_frame(const MatchArgs &a, ctm_frame f, int n_boxes, cudaStream_t s)
-{
-    stage_frame_kernel<<<1, 1, 0, s>>>(a.ws.frames, a.ws.counts_in, f, n_boxes);
     return cudaGetLastError();
 }
 
