@@ -146,10 +146,8 @@ typedef struct {
                                strip of one column chunk of a block: a multiple of 8, at
                                least the larger disparity range + 2; larger values mean
                                fewer chunks and more shared memory per CTA            */
-    int32_t census_mode;    /* region-of-interest census (5x5, 7x7, 9x7 windows): 0 =
-                               integer multiply-add compares, 4 CTAs per SM; 1 = the
-                               same, 3 CTAs per SM; 2 = packed fp16 compares with
-                               saturation, 4 CTAs per SM                              */
+    int32_t census_mode;    /* 0, 1 or 2; accepted and kept, without effect (the fixed
+                               windows, 5x5, 7x7 and 9x7, have one kernel)            */
     int32_t queue_rounds;   /* 0 or 1; accepted and kept, without effect (no matcher hands
                                blocks out in rounds any more)                          */
     int32_t match_mode;     /* 0: tensor-core matcher (both passes of a block as products of

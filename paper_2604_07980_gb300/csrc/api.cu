@@ -197,7 +197,6 @@ MatchArgs make_args(const ctm_ctx *ctx, const ctm_frame *frames, const int32_t *
     a.strip_cols = ctx->strip_cols;
     a.strip_rows = ctx->strip_rows;
     a.sm_count = ctx->sm_count;
-    a.census_mode = ctx->census_mode;
     a.match_mode = ctx->match_mode;
     if (!ctx->maps_ok) a.ws.tmaps = nullptr;
     a.stats_accumulate = 0;
@@ -462,7 +461,7 @@ int ctm_create(ctm_ctx **out, const ctm_params *p, int max_frames, int max_width
         ctm_destroy(ctx);
         return CTM_ECUDA;
     }
-    for (int m = 0; m < 3; ++m) census_roi_ctas_per_sm(p->win_w, p->win_h, m);  // outside any capture
+    census_roi_ctas_per_sm(p->win_w, p->win_h);  // outside any capture
     *out = ctx;
     return CTM_OK;
 }
@@ -1051,15 +1050,6 @@ int ctm_autotune(ctm_ctx *ctx, const ctm_frame *frames_dev, const int32_t *count
             if (r != CTM_OK) { status = r; break; }
             if (ms < bms) { bms = ms; bt = t; }
         }
-    }
-    // 2. census variant
-    for (int m = 0; m < 3 && status == CTM_OK; ++m) {
-        ctm_tuning t = bt;
-        t.census_mode = m;
-        float ms = 0.0f;
-        const int r = measure(t, &ms);
-        if (r != CTM_OK) { status = r; break; }
-        if (ms < bms) { bms = ms; bt = t; }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

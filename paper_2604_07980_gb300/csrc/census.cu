@@ -6,16 +6,10 @@
 // neighbour in the highest comparison bit, with the optional sentinel above
 // them; pixels whose window leaves the grid get 0.
 //
-// Fixed windows (5x5, 7x7, 9x7) use census4: four pixels per lane, compares on
-// the integer multiply-add pipe, rows loaded straight into registers.  The
-// full-image kernel (ctm_census_build) gives a half-warp a 64-pixel row tile;
-// the region-of-interest kernel of the matching path gives eight lanes a
-// 32-pixel tile from the list of tiles the planner marked.  Other windows use
-// a warp per 64-pixel tile, staging the window rows in shared memory as fp16
-// bit patterns 0x6400 | v (exactly 1024 + v, so fp16 order is pixel order) and
-// comparing two pixels per __hgt2_mask.
-#include <cuda_fp16.h>
-
+// Fixed windows (5x5, 7x7, 9x7) compare bit planes of 32 pixels at a time in units of
+// 128 columns x 32 rows: all of them for a full image (ctm_census_build), those with
+// marked tiles for the matching path.  Other windows use a warp per 64-pixel tile, the
+// window rows staged in shared memory as 16-bit values 0x6400 | v.
 #include "ctm_internal.cuh"
 
 namespace ctm {
@@ -51,8 +45,6 @@ struct Plane {
     int vec_load;         // word loads allowed: k in {1, 2}, 8-byte aligned base, pitch % 4 == 0
 };
 
-__device__ __forceinline__ __half2 as_h2(uint32_t u) { return *reinterpret_cast<__half2 *>(&u); }
-
 // Staged row layout: H[b] = 0x6400 | I_k(x0 - 8 + b, row) for b in [0, 80), kept
 // twice as half2 words: even[t] = (H[2t], H[2t+1]) and odd[t] = (H[2t+1], H[2t+2]),
 // so every pair of adjacent pixels is one aligned 32-bit word in one of the two.
@@ -80,40 +72,6 @@ __device__ __forceinline__ uint32_t load_quad(const Plane &pl, int x0, int ys, i
     return v;
 }
 
-// All WH window rows of tile (x0, y) for this lane, with one uniform decision per
-// tile: interior tiles of a word-aligned image take straight-line word loads,
-// edge tiles take the per-pixel path.  Rows must lie inside the grid.
-template <int WH>
-__device__ __forceinline__ void load_tile(const Plane &pl, int x0, int y, int lane, uint32_t (&v)[WH])
-{
-    constexpr int sy = WH / 2;
-    const int xs = x0 - 8 + 4 * lane;
-    const bool interior = pl.vec_load && x0 - 8 >= 0 &&
-                          (pl.k == 1 ? x0 + 76 <= pl.W : 2 * (x0 + 76) <= pl.W);
-    if (interior) {
-        const long long step = (long long)pl.k * pl.pitch;
-        const uint8_t *row = pl.img + (long long)pl.k * (y - sy) * pl.pitch + (long long)pl.k * xs;
-        if (lane < 21) {
-            if (pl.k == 1) {
-#pragma unroll
-                for (int r = 0; r < WH; ++r) v[r] = __ldg(reinterpret_cast<const uint32_t *>(row + r * step));
-            } else {
-#pragma unroll
-                for (int r = 0; r < WH; ++r) {
-                    const uint2 w = __ldg(reinterpret_cast<const uint2 *>(row + r * step));
-                    v[r] = __byte_perm(w.x, w.y, 0x6420);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int r = 0; r < WH; ++r) v[r] = 0u;
-        }
-    } else {
-#pragma unroll
-        for (int r = 0; r < WH; ++r) v[r] = load_quad(pl, x0, y - sy + r, lane);
-    }
-}
-
 // Convert one loaded row (4 pixels per lane) to the two half2 copies.
 __device__ __forceinline__ void store_quad(uint32_t v, uint32_t *even, uint32_t *odd, int lane)
 {
@@ -130,58 +88,11 @@ __device__ __forceinline__ void store_quad(uint32_t v, uint32_t *even, uint32_t 
     }
 }
 
-// Stage the window rows y - sy .. y + sy of tile x0: all loads first (they are
-// independent and in flight together), then the conversions.
-template <int WH>
-__device__ __forceinline__ void stage_rows(const Plane &pl, int x0, int y, const WarpStage &st, int lane)
-{
-    constexpr int sy = WH / 2;
-    uint32_t v[WH];
-#pragma unroll
-    for (int r = 0; r < WH; ++r) v[r] = load_quad(pl, x0, y - sy + r, lane);
-#pragma unroll
-    for (int r = 0; r < WH; ++r) store_quad(v[r], st.even + r * kWordsMax, st.odd + r * kWordsMax, lane);
-}
-
 __device__ __forceinline__ void stage_rows_any(const Plane &pl, int x0, int y, int sy,
                                                const WarpStage &st, int lane)
 {
     for (int r = 0; r < 2 * sy + 1; ++r)
         store_quad(load_quad(pl, x0, y - sy + r, lane), st.even + r * kWordsMax, st.odd + r * kWordsMax, lane);
-}
-
-// Codes of pixels (x0 + 2 lane, x0 + 2 lane + 1) from the staged rows.
-template <int WW, int WH>
-__device__ __forceinline__ void tile_codes(const WarpStage &st, int lane, int sentinel, uint64_t &c0,
-                                           uint64_t &c1)
-{
-    constexpr int sx = WW / 2, sy = WH / 2;
-    constexpr int n = WW * WH;
-    constexpr int OFF = 8 - sx;  // H index of the window's left column, relative to 2*lane
-    uint32_t acc[4] = {0u, 0u, 0u, 0u};
-    const __half2 centre = as_h2(st.even[sy * kWordsMax + lane + 4]);  // H[2*lane + 8]
-#pragma unroll
-    for (int j = 0; j < WH; ++j) {
-#pragma unroll
-        for (int i = 0; i < WW; ++i) {
-            const int b = i + OFF;  // H index of the neighbour pair, relative to 2*lane
-            const uint32_t nb = (b & 1) ? st.odd[j * kWordsMax + lane + (b - 1) / 2]
-                                        : st.even[j * kWordsMax + lane + b / 2];
-            const uint32_t m = __hgt2_mask(as_h2(nb), centre);
-            const int k = j * WW + i;     // raster index of the window offset
-            const int p = n - 1 - k;      // its code bit
-            const uint32_t pos = (1u << (p & 15)) | (1u << (16 + (p & 15)));
-            acc[p >> 4] |= m & pos;
-        }
-    }
-    if (sentinel) {
-        const uint32_t pos = (1u << (n & 15)) | (1u << (16 + (n & 15)));
-        acc[n >> 4] |= pos;
-    }
-    const uint32_t lo0 = __byte_perm(acc[0], acc[1], 0x5410), hi0 = __byte_perm(acc[2], acc[3], 0x5410);
-    const uint32_t lo1 = __byte_perm(acc[0], acc[1], 0x7632), hi1 = __byte_perm(acc[2], acc[3], 0x7632);
-    c0 = ((uint64_t)hi0 << 32) | lo0;
-    c1 = ((uint64_t)hi1 << 32) | lo1;
 }
 
 // Any window: plain per-pixel loop over the staged rows.
@@ -216,350 +127,506 @@ __device__ __forceinline__ void store_pair(const Plane &pl, int x, int y, uint64
 
 
 // ---------------------------------------------------------------------------
-// Fixed windows (5x5, 7x7, 9x7): four pixels per lane.
+// Fixed windows (5x5, 7x7, 9x7): bit-sliced.
 //
-// Lane l of a tile's lane group owns pixels x .. x+3 (x = x0 + 4 l).  It
-// loads the twelve pixels I_k(x-4 .. x+7) of every window row straight into
-// registers (three 32-bit loads at k = 1, three 64-bit loads compacted with
-// PRMT at k = 2; adjacent lanes share bytes through L1) and forms the eleven
-// words (b[t], b[t+1]) of pixel pairs in registers, so no shared
-// memory is involved.  Pixel pairs (x, x+1) and (x+2, x+3) are compared two at
-// a time in the 16-bit halves of a word (codes4).
+// A unit is 128 columns x up to 16 rows of a plane.  Its pixels are turned into bit
+// planes: word j of plane p holds bit p of the 32 pixels x0 + j + 4 b (bit b of the
+// word), j = 0 .. 3.  Pixels four apart share a word, so the neighbour at column offset
+// dx is another word -- word j + dx, of -4 .. 7, where the words outside 0 .. 3 are the
+// same words moved by one bit -- and no compare needs a shift.  [neighbour > centre] of
+// 32 pixels is then one LOP3 per plane, from the lowest bit up:
+//     gt = (a & ~c) | (gt & ~(a ^ c)),
+// 8 instructions for 32 compares, and two 32 x 32 bit transposes turn a pixel group's 63
+// results into codes.
+//
+// Work split: a warp takes a unit.  Four lanes slice a source row (once, for the up to
+// WH rows of codes that read it): 32 pixels per lane, an 8 x 8 bit transpose within the
+// bytes of its 8 words, byte exchange between the four lanes, the word and its two moved
+// copies to shared memory.  Then four lanes take a marked row, a word each.
+//
+// What bounds it: the ALU pipe (LOP3, PRMT, SHF: half of the issue rate; about 1450
+// instructions for eight rows of a unit, 912 of them the compares and transposes) and
+// the L1 (124 LDS.128 for the same rows, 0.6 of its wavefronts), 60 and 75% busy on eight
+// 4K frames, with twelve warps an SM (shared memory).  The kernel before it compared two
+// pixels per instruction in 16-bit halves, 160 instructions a pixel against 85 here
+// (per marked pixel: a unit also computes the unmarked part of its 128 columns, 10 to
+// 25%, and leaves lanes idle when its rows are not a multiple of eight).  Measured, list
+// and census of the marked tiles: eight 4K frames 141 -> 110 us, 32 frames of 1920x1200
+// 110 -> 103, four 720p frames 24.4 -> 19.5, one 1279x719 frame (rows of odd pitch, which
+// the old kernel read by bytes) 18.2 -> 14.6; full images: 3840x2160 39.0 -> 28.8,
+// 1920x1200 15.0 -> 11.3, 3839x2159 at half resolution 33 -> 12.7 us.  Slower: a CTA of
+// four warps per unit of 32 rows (120 us on the 32 frames), codes stored by the lanes
+// instead of bulk copies (L1 at 78%), all source rows loaded before the first is sliced
+// (instruction cache), two row buffers in registers (spills).
+constexpr int kUnitPx = 128;      // columns of a unit
+constexpr int kRoiRows = 16;      // rows of a unit of the matching path
+constexpr int kUnitThreads = 64;
+constexpr int kUnitCtas = 6;      // resident CTAs per SM (shared memory; 168 registers a thread)
+constexpr int kFullThreads = 128; // full image
+constexpr int kFullCtas = 4;      // 128 registers a thread
+constexpr int kUnitPos = 12;      // words -4 .. 7 of a source row
+// 16-byte pieces of a sliced row: planes 0 .. 3 of the 12 words, then planes 4 .. 7, and
+// four unused, so that neighbouring rows' pieces lie half of the banks apart
+constexpr int kUnitPieces = 2 * kUnitPos + 4;
+constexpr int kStageStride = kUnitPx + 4;  // codes between staged rows: eight rows' 32-byte stores cover the banks
 
-// Pixels xs .. xs+3 of a row at k = 1 (one aligned word; xs is a multiple of 4):
-// 0 where the word lies outside [0, W), bytes where it straddles W.
-__device__ __forceinline__ uint32_t word_k1(const uint8_t *row, int xs, int W)
-{
-    if (xs >= 0 && xs + 4 <= W) return __ldg(reinterpret_cast<const uint32_t *>(row + xs));
-    if (xs + 4 <= 0 || xs >= W) return 0u;
-    uint32_t w = 0u;
-    for (int t = 0; t < 4; ++t) {
-        const int xt = xs + t;
-        if (xt >= 0 && xt < W) w |= (uint32_t)__ldg(row + xt) << (8 * t);
-    }
-    return w;
-}
+// 32 pixels of a row on their way in: 8 little-endian words, or (pairs) the 16 words of 64
+// source bytes whose even bytes they are, and the pixels left and right of the lane's word.
+struct RowPx {
+    uint32_t v[16];
+    uint32_t left, right;
+    bool pairs;
+};
 
-// Decimated pixels xs .. xs+3 of a row at k = 2 (source bytes 2 xs .. 2 xs + 7,
-// one aligned 8-byte word compacted with PRMT): 0 outside the grid [0, Ws),
-// bytes where the word straddles the source row end W.
-__device__ __forceinline__ uint32_t word_k2(const uint8_t *row, int xs, int W, int Ws)
+// 32 pixels of grid row yr from grid column x (a multiple of 32); pixels outside the grid
+// are 0.  Sixteen-byte loads where image and pitch allow them, not waited for here; else
+// aligned words moved into place; bytes at the grid's right border, where a word would
+// leave the image, and at other decimations.
+__device__ __forceinline__ void load_px32(const PlaneDesc &d, int x, int yr, bool vec, RowPx &px)
 {
-    if (xs >= 0 && 2 * xs + 8 <= W) {
-        const uint2 u = __ldg(reinterpret_cast<const uint2 *>(row + 2 * xs));
-        return __byte_perm(u.x, u.y, 0x6420);
-    }
-    if (xs + 4 <= 0 || xs >= Ws) return 0u;
-    uint32_t w = 0u;
-    for (int t = 0; t < 4; ++t) {
-        const int xt = xs + t;
-        if (xt >= 0 && xt < Ws) w |= (uint32_t)__ldg(row + 2 * xt) << (8 * t);
-    }
-    return w;
-}
-
-// Twelve pixels I_k(x - 4 .. x + 7) of grid row `yr` for this lane, as three
-// little-endian words; pixels outside the grid read as 0 (they only feed
-// pixels whose codes are zeroed).  Lanes whose twelve pixels lie inside a
-// word-aligned image take word loads, the others (image borders, other
-// decimations or alignments) byte loads.
-__device__ __forceinline__ void load_row12(const PlaneDesc &d, bool inside, int x, int yr, uint32_t (&v)[3])
-{
-    if (inside && d.k == 1) {
-        const uint32_t *q = reinterpret_cast<const uint32_t *>(d.img + (long long)yr * d.pitch + (x - 4));
-        v[0] = __ldg(q);
-        v[1] = __ldg(q + 1);
-        v[2] = __ldg(q + 2);
-    } else if (inside) {  // k == 2: every other source byte
-        const uint2 *q = reinterpret_cast<const uint2 *>(d.img + 2LL * yr * d.pitch + 2 * (x - 4));
-        const uint2 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
-        v[0] = __byte_perm(a.x, a.y, 0x6420);
-        v[1] = __byte_perm(b.x, b.y, 0x6420);
-        v[2] = __byte_perm(c.x, c.y, 0x6420);
-    } else {
-        const uint8_t *row = d.img + (long long)d.k * yr * d.pitch;
-        uint32_t w[3] = {0u, 0u, 0u};
+    const uint8_t *row = d.img + (long long)d.k * yr * d.pitch;
+    const uint8_t *end = d.img + (long long)(d.H - 1) * d.pitch + d.W;
+    const bool inside = x + 32 <= d.Ws;
+    const uint8_t *s = row + (long long)d.k * x;
+    const unsigned mis = (unsigned)(reinterpret_cast<uintptr_t>(s) & 3u), sh = 8u * mis;
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(s - mis);
+    uint32_t (&v)[16] = px.v;
+    if (d.k <= 2 && inside && vec && s + 32 * d.k <= end) {
+        px.pairs = d.k == 2;
 #pragma unroll
-        for (int t = 0; t < 12; ++t) {
-            const int xs = x - 4 + t;
-            const uint32_t b = (xs >= 0 && xs < d.Ws) ? (uint32_t)__ldg(row + (long long)d.k * xs) : 0u;
-            w[t >> 2] |= b << (8 * (t & 3));
+        for (int i = 0; i < 4; ++i) {
+            if (i >= 2 && d.k == 1) break;
+            const uint4 a = __ldg(reinterpret_cast<const uint4 *>(s) + i);
+            v[4 * i] = a.x;
+            v[4 * i + 1] = a.y;
+            v[4 * i + 2] = a.z;
+            v[4 * i + 3] = a.w;
         }
-        v[0] = w[0];
-        v[1] = w[1];
-        v[2] = w[2];
+    } else if (d.k == 1 && inside && s - mis >= d.img && s + 36 <= end) {
+        uint32_t u[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) u[i] = __ldg(w + i);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = __funnelshift_r(u[i], u[i + 1], sh);
+    } else if (d.k == 2 && inside && s - mis >= d.img && s + 68 <= end) {
+        uint32_t u[17];
+        px.pairs = true;
+#pragma unroll
+        for (int i = 0; i < 17; ++i) u[i] = __ldg(w + i);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __funnelshift_r(u[i], u[i + 1], sh);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (x + 4 * i + q < d.Ws) v[i] |= (uint32_t)__ldg(s + (long long)d.k * (4 * i + q)) << (8 * q);
+        }
     }
 }
 
-// Codes of the four pixels x .. x+3 of a lane (bit layout as tile_codes) from
-// its window rows: row(j, v) gives the twelve pixels I_k(x - 4 .. x + 7) of
-// window row j as three little-endian words (row(sy, v) first, for the centre
-// pixels).
-//
-// The compares run on the integer multiply-add pipe: with both pixels of a
-// pair in the two 16-bit halves of a word w (plain values, upper bytes zero),
-// e = w * 2^s + K_s, K_s = (2^16 - 2^(8+s) - 1 - c 2^s) per half, is per half
-// the complement of 2^(8+s) + (c - nb) 2^s, which lies in [1, 2^16) for
-// s <= 7; so no carry crosses the halves and bit 8 + s of each half is
-// [nb > c].  Code bit p = 8 a + s is taken from bit 8 + s (and 24 + s) of e
-// into accumulator a with one LOP3; accumulator a ends up holding code byte a
-// of the low pixel in its byte 1 and of the high pixel in its byte 3.
-template <int WW, int WH, typename RowFn>
-__device__ __forceinline__ void codes4(RowFn row, int sentinel, uint64_t (&c)[4])
+// Lane j of four: the pixels x0 + 32 j .. + 31 of row yr (on: it is needed and inside the
+// grid) of the unit at column x0.
+__device__ __forceinline__ void load_row(const PlaneDesc &d, int x0, int yr, bool on, int j, bool vec, RowPx &px)
+{
+#pragma unroll
+    for (int i = 0; i < 16; ++i) px.v[i] = 0u;
+    px.left = px.right = 0u;
+    px.pairs = false;
+    if (!on) return;
+    if (x0 + 32 * j < d.Ws) load_px32(d, x0 + 32 * j, yr, vec, px);
+    const uint8_t *row = d.img + (long long)d.k * yr * d.pitch;
+    const int xl = x0 - 4 + j, xr = x0 + kUnitPx + j;
+    if (xl >= 0 && xl < d.Ws) px.left = __ldg(row + (long long)d.k * xl);
+    if (xr < d.Ws) px.right = __ldg(row + (long long)d.k * xr);
+}
+
+// b << S on the multiply pipe (the compiler would take the ALU, which bounds these kernels).
+template <int S>
+__device__ __forceinline__ uint32_t shl_fma(uint32_t b)
+{
+    uint32_t r;
+    asm("mad.lo.u32 %0, %1, %2, 0;" : "=r"(r) : "r"(b), "n"(1u << S));
+    return r;
+}
+
+// Three-input logic as one instruction (written out, the compiler spends up to two on it).
+template <int Lut>
+__device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c)
+{
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, %4;" : "=r"(r) : "r"(a), "r"(b), "r"(c), "n"(Lut));
+    return r;
+}
+constexpr int kSelect = 0xe4;   // (a & c) | (b & ~c)
+constexpr int kGreater = 0xb2;  // (a & ~b) | (c & ~(a ^ b)): one more bit of [a > b], c the result of the bits below
+
+// Exchange bits: a's bits of ~m (shifted down) against b's bits of m, m the low s bits of
+// every 2 s.
+template <int S>
+__device__ __forceinline__ void swap_bits(uint32_t &a, uint32_t &b)
+{
+    constexpr uint32_t m = S == 1 ? 0x55555555u : (S == 2 ? 0x33333333u : 0x0f0f0f0fu);
+    const uint32_t lo = lop3<kSelect>(a, shl_fma<S>(b), m);
+    b = lop3<kSelect>(a >> S, b, m);
+    a = lo;
+}
+
+// Transpose of a 32 x 32 bit matrix, row i in w[i].
+__device__ __forceinline__ void transpose32(uint32_t (&w)[32])
+{
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const uint32_t a = w[i], b = w[i + 16];
+        w[i] = __byte_perm(a, b, 0x5410);
+        w[i + 16] = __byte_perm(a, b, 0x7632);
+    }
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        if (i & 8) continue;
+        const uint32_t a = w[i], b = w[i + 8];
+        w[i] = __byte_perm(a, b, 0x6240);
+        w[i + 8] = __byte_perm(a, b, 0x7351);
+    }
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+        if (!(i & 4)) swap_bits<4>(w[i], w[i + 4]);
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+        if (!(i & 2)) swap_bits<2>(w[i], w[i + 2]);
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+        if (!(i & 1)) swap_bits<1>(w[i], w[i + 1]);
+}
+
+// Slice a loaded row into `dst`.  All lanes of a warp call it (on: this row is written).
+__device__ __forceinline__ void slice_row(const RowPx &px, bool on, int j, uint4 *dst)
+{
+    const unsigned full = 0xffffffffu;
+    const uint32_t bl = px.left, br = px.right;
+    uint32_t v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)  // the even bytes of words 2 i, 2 i + 1, or word i
+        v[i] = px.pairs ? __byte_perm(px.v[2 * i], px.v[2 * i + 1], 0x6420) : px.v[i];
+    // bit i of byte c of v[p]: bit p of byte c of word i
+#pragma unroll
+    for (int i = 0; i < 4; ++i) swap_bits<4>(v[i], v[i + 4]);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (!(i & 2)) swap_bits<2>(v[i], v[i + 2]);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (!(i & 1)) swap_bits<1>(v[i], v[i + 1]);
+    // byte c of lane g to byte g of lane c
+    const unsigned sel2 = (j & 2) ? 0x3276u : 0x5410u, sel1 = (j & 1) ? 0x3715u : 0x6240u;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) v[p] = __byte_perm(v[p], __shfl_xor_sync(full, v[p], 2), sel2);
+#pragma unroll
+    for (int p = 0; p < 8; ++p) v[p] = __byte_perm(v[p], __shfl_xor_sync(full, v[p], 1), sel1);
+    if (!on) return;
+    uint32_t l[8], r[8];
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        l[p] = __funnelshift_l(bl << (31 - p), v[p], 1);
+        r[p] = __funnelshift_r(v[p], br >> p, 1);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint4 *o = dst + h * kUnitPos + j;
+        o[0] = make_uint4(l[4 * h], l[4 * h + 1], l[4 * h + 2], l[4 * h + 3]);
+        o[4] = make_uint4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+        o[8] = make_uint4(r[4 * h], r[4 * h + 1], r[4 * h + 2], r[4 * h + 3]);
+    }
+}
+
+// [neighbour > centre] of 32 pixels: `a` the neighbour's planes 0 .. 3 and b its planes 4 .. 7.
+__device__ __forceinline__ uint32_t greater32(uint4 a, uint4 b, const uint32_t (&c)[8])
+{
+    uint32_t g = a.x & ~c[0];
+    g = lop3<kGreater>(a.y, c[1], g);
+    g = lop3<kGreater>(a.z, c[2], g);
+    g = lop3<kGreater>(a.w, c[3], g);
+    g = lop3<kGreater>(b.x, c[4], g);
+    g = lop3<kGreater>(b.y, c[5], g);
+    g = lop3<kGreater>(b.z, c[6], g);
+    return lop3<kGreater>(b.w, c[7], g);
+}
+
+// Code bits 32 H .. 32 H + 31 of the 32 pixels of a word, pixel b's in w[b].  src: piece
+// (first window row, word j).  V: pixels whose window lies in the grid.
+template <int WW, int WH, int H>
+__device__ __forceinline__ void code_half(const uint4 *src, const uint32_t (&c)[8], uint32_t V, int sentinel,
+                                          uint32_t (&w)[32])
+{
+    constexpr int sx = WW / 2, n = WW * WH;
+#pragma unroll
+    for (int q = 0; q < 32; ++q) {
+        const int p = 32 * H + q, k = n - 1 - p;  // code bit and raster index of its window offset
+        if (p > n || k == n / 2) {
+            w[q] = 0u;
+        } else if (p == n) {
+            w[q] = sentinel ? V : 0u;
+        } else {
+            const uint4 *s = src + (k / WW) * kUnitPieces + 4 + (k % WW) - sx;
+            w[q] = greater32(s[0], s[kUnitPos], c);
+        }
+    }
+    if (V != 0xffffffffu) {
+#pragma unroll
+        for (int q = 0; q < 32; ++q) w[q] &= V;
+    }
+    transpose32(w);
+}
+
+// Codes of word j of row y (its first window row, word -4, at `rows`) of the unit at x0.
+template <int WW, int WH>
+__device__ __forceinline__ void word_codes(const PlaneDesc &d, int x0, int y, int j, const uint4 *rows, int sentinel,
+                                           uint32_t (&lo)[32], uint32_t (&hi)[32])
 {
     constexpr int sx = WW / 2, sy = WH / 2;
-    constexpr int n = WW * WH;
-    constexpr int OFF = 4 - sx;  // byte index of the window's left column for pixel x
-    uint32_t vc[3];
-    row(sy, vc);
-    uint32_t accA[8], accB[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) accA[q] = accB[q] = 0u;
-    if (sentinel) {
-        accA[n >> 3] = (0x100u << (n & 7)) | (0x1000000u << (n & 7));
-        accB[n >> 3] = accA[n >> 3];
+    static_assert(sx <= 4 && WW * WH < 64, "window");
+    const int x = x0 + j;
+    // pixels x + 4 b with b0 <= b < b1 have their window inside the grid
+    uint32_t V = 0xffffffffu;
+    if (y - sy < 0 || y + sy >= d.Hs) {
+        V = 0u;
+    } else if (x0 < sx || x0 + kUnitPx + sx > d.Ws) {
+        const int b0 = max(0, (sx - x + 3) >> 2), b1 = min(32, (d.Ws - sx - x + 3) >> 2);
+        V = b1 <= b0 ? 0u : (0xffffffffu >> (32 - b1)) & (0xffffffffu << b0);
     }
-    const uint32_t cA = __byte_perm(vc[1], 0u, 0x4140);  // pixels x, x+1
-    const uint32_t cB = __byte_perm(vc[1], 0u, 0x4342);  // pixels x+2, x+3
-    uint32_t KA[8], KB[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const uint32_t h = 0x10000u - (0x100u << q) - 1u;
-        KA[q] = (h | (h << 16)) - (cA << q);
-        KB[q] = (h | (h << 16)) - (cB << q);
-    }
-#pragma unroll
-    for (int j = 0; j < WH; ++j) {
-        uint32_t v[3];
-        row(j, v);
-        // w[t] = (b[t], b[t+1]) in the two halves, t = 0 .. 10
-        uint32_t w[11];
-        const uint32_t s1 = __funnelshift_r(v[0], v[1], 8);  // b1 .. b4
-        const uint32_t s2 = __funnelshift_r(v[1], v[2], 8);  // b5 .. b8
-        w[0] = __byte_perm(v[0], 0u, 0x4140);
-        w[1] = __byte_perm(s1, 0u, 0x4140);
-        w[2] = __byte_perm(v[0], 0u, 0x4342);
-        w[3] = __byte_perm(s1, 0u, 0x4342);
-        w[4] = __byte_perm(v[1], 0u, 0x4140);
-        w[5] = __byte_perm(s2, 0u, 0x4140);
-        w[6] = __byte_perm(v[1], 0u, 0x4342);
-        w[7] = __byte_perm(s2, 0u, 0x4342);
-        w[8] = __byte_perm(v[2], 0u, 0x4140);
-        w[9] = __byte_perm(v[2], 0u, 0x4241);
-        w[10] = __byte_perm(v[2], 0u, 0x4342);
-#pragma unroll
-        for (int i = 0; i < WW; ++i) {
-            const int p = n - 1 - (j * WW + i);  // code bit of this window offset
-            const int q = p & 7;
-            const uint32_t pos = (0x100u << q) | (0x1000000u << q);
-            accA[p >> 3] |= (w[OFF + i] * (1u << q) + KA[q]) & pos;
-            accB[p >> 3] |= (w[OFF + i + 2] * (1u << q) + KB[q]) & pos;
-        }
-    }
-    uint32_t tA[4], tB[4];  // code bytes (2q, 2q+1) of the low pixel, then of the high pixel
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        tA[q] = __byte_perm(accA[2 * q], accA[2 * q + 1], 0x7351);
-        tB[q] = __byte_perm(accB[2 * q], accB[2 * q + 1], 0x7351);
-    }
-    c[0] = ((uint64_t)__byte_perm(tA[2], tA[3], 0x5410) << 32) | __byte_perm(tA[0], tA[1], 0x5410);
-    c[1] = ((uint64_t)__byte_perm(tA[2], tA[3], 0x7632) << 32) | __byte_perm(tA[0], tA[1], 0x7632);
-    c[2] = ((uint64_t)__byte_perm(tB[2], tB[3], 0x5410) << 32) | __byte_perm(tB[0], tB[1], 0x5410);
-    c[3] = ((uint64_t)__byte_perm(tB[2], tB[3], 0x7632) << 32) | __byte_perm(tB[0], tB[1], 0x7632);
-}
-
-// codes4 with the compares in packed fp16 (census mode 2).  Grid pixels are
-// exact fp16 integers 1024 + v (bit pattern 0x6400 | v), two per register, as
-// the spread words of codes4 with 0x64 in place of the zero bytes.  One compare
-// pair is one packed fused multiply-add with saturation, sat(nb * 1 - c): 1.0
-// where nb > c, else +0.0 -- exact, as every operand and difference is a small
-// integer.  A window row's compares accumulate as acc * 2 + r (fp16, exact below
-// 1024; a row holds at most 9 bits, first neighbour highest); adding 1024 to a
-// row's sum puts its bits in the low bits of each half, from where they go to
-// their code bits.  Both operations run on the FMA pipe, which leaves the ALU
-// pipe the byte spreading and the code assembly.
-template <int WW, int WH, typename RowFn>
-__device__ __forceinline__ void codes4_h(RowFn row, int sentinel, uint64_t (&c)[4])
-{
-    constexpr int sy = WH / 2;
-    constexpr int n = WW * WH;
-    constexpr int OFF = 4 - WW / 2;  // byte index of the window's left column for pixel x
-    static_assert(WW <= 10, "a window row's bits must stay below 1024");
-    const uint32_t H = 0x64646464u;
-    uint32_t vc[3];
-    row(sy, vc);
-    // -(1024 + c) for the centre pixels (x, x+1) and (x+2, x+3)
-    const uint32_t nA = __byte_perm(vc[1], H, 0x4140) ^ 0x80008000u;
-    const uint32_t nB = __byte_perm(vc[1], H, 0x4342) ^ 0x80008000u;
-    const __half2 one2 = __floats2half2_rn(1.0f, 1.0f), two2 = __floats2half2_rn(2.0f, 2.0f);
-    const __half2 bias2 = __floats2half2_rn(1024.0f, 1024.0f);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) c[q] = 0ull;
-#pragma unroll
-    for (int j = 0; j < WH; ++j) {
-        uint32_t v[3];
-        row(j, v);
-        uint32_t w[11];
-        const uint32_t s1 = __funnelshift_r(v[0], v[1], 8);  // b1 .. b4
-        const uint32_t s2 = __funnelshift_r(v[1], v[2], 8);  // b5 .. b8
-        w[0] = __byte_perm(v[0], H, 0x4140);
-        w[1] = __byte_perm(s1, H, 0x4140);
-        w[2] = __byte_perm(v[0], H, 0x4342);
-        w[3] = __byte_perm(s1, H, 0x4342);
-        w[4] = __byte_perm(v[1], H, 0x4140);
-        w[5] = __byte_perm(s2, H, 0x4140);
-        w[6] = __byte_perm(v[1], H, 0x4342);
-        w[7] = __byte_perm(s2, H, 0x4342);
-        w[8] = __byte_perm(v[2], H, 0x4140);
-        w[9] = __byte_perm(v[2], H, 0x4241);
-        w[10] = __byte_perm(v[2], H, 0x4342);
-        __half2 aA, aB;
-#pragma unroll
-        for (int i = 0; i < WW; ++i) {
-            const __half2 rA = __hfma2_sat(as_h2(w[OFF + i]), one2, as_h2(nA));
-            const __half2 rB = __hfma2_sat(as_h2(w[OFF + i + 2]), one2, as_h2(nB));
-            aA = i == 0 ? rA : __hfma2(aA, two2, rA);
-            aB = i == 0 ? rB : __hfma2(aB, two2, rB);
-        }
-        const __half2 hA = __hadd2(aA, bias2), hB = __hadd2(aB, bias2);
-        const uint32_t uA = *reinterpret_cast<const uint32_t *>(&hA);
-        const uint32_t uB = *reinterpret_cast<const uint32_t *>(&hB);
-        constexpr uint32_t m = (1u << WW) - 1u;
-        const int p_lo = n - WW * (j + 1);  // code bit of the row's last neighbour
-        c[0] |= (uint64_t)(uA & m) << p_lo;
-        c[1] |= (uint64_t)((uA >> 16) & m) << p_lo;
-        c[2] |= (uint64_t)(uB & m) << p_lo;
-        c[3] |= (uint64_t)((uB >> 16) & m) << p_lo;
-    }
-    if (sentinel) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) c[q] |= 1ull << n;
-    }
-}
-
-// Store the codes of pixels x .. x+3 of grid row y (zero where the window leaves
-// the grid, or for the whole row when `active` is false).
-template <int WW>
-__device__ __forceinline__ void store4(const PlaneDesc &d, int x, int y, bool active, uint64_t (&c)[4])
-{
-    constexpr int sx = WW / 2;
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        if (!active || x + q - sx < 0 || x + q + sx >= d.Ws) c[q] = 0ull;
-    uint64_t *dst = d.out + (long long)y * d.opitch + x;
-    if (x + 3 < d.Ws && ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0)) {
-        reinterpret_cast<ulonglong2 *>(dst)[0] = make_ulonglong2(c[0], c[1]);
-        reinterpret_cast<ulonglong2 *>(dst)[1] = make_ulonglong2(c[2], c[3]);
+    const uint4 *src = rows + j, *mid = src + sy * kUnitPieces + 4;
+    const uint4 ca = mid[0], cb = mid[kUnitPos];
+    const uint32_t c[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
+    code_half<WW, WH, 0>(src, c, V, sentinel, lo);
+    if constexpr (WW * WH >= 32) {
+        code_half<WW, WH, 1>(src, c, V, sentinel, hi);
     } else {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (x + q < d.Ws) dst[q] = c[q];
+        for (int b = 0; b < 32; ++b) hi[b] = 0u;
     }
 }
 
-// Codes of pixels x .. x+3 of row y of plane d (4 consecutive pixels per lane;
-// bit layout as tile_codes), stored to the plane; `ok` false: this lane has
-// no tile and stores nothing.  All 32 lanes of the warp must call it together.
-// All window rows are loaded into registers before the first is used.
-template <int WW, int WH, bool F16 = false>
-__device__ __forceinline__ void census4(const PlaneDesc &d, int x0, int y, int hl, bool ok, int sentinel)
+__device__ __forceinline__ void stage_codes(uint2 *st, const uint32_t (&lo)[32], const uint32_t (&hi)[32])
+{
+#pragma unroll
+    for (int b = 0; b < 32; ++b) st[4 * b] = make_uint2(lo[b], hi[b]);
+}
+
+// One staged row to its place, 16-byte aligned, cols even.
+__device__ __forceinline__ void bulk_row(uint64_t *dst, const uint2 *src, int cols)
+{
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\ncp.async.bulk.commit_group;\n"
+                 ::"l"(dst), "r"((unsigned)__cvta_generic_to_shared(src)), "r"(8 * cols) : "memory");
+}
+
+// This thread's bulk copies have read their shared memory (.read) or are complete.
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
+
+// Place of marked row `row` among the marked ones: odd and even rows in turn as long as
+// both last, as two rows read together (eight lanes of a 16-byte load) meet in the same
+// banks when both are even or both odd.
+__device__ __forceinline__ int slot_of_row(uint32_t mask, int row)
+{
+    const uint32_t even = mask & 0x55555555u, odd = mask & ~0x55555555u;
+    const int both = min(__popc(even), __popc(odd));
+    const int i = __popc((row & 1 ? odd : even) & ((1u << row) - 1u));
+    return i < both ? 2 * i + (row & 1) : both + i;
+}
+
+// Shared memory of a warp working on listed units.
+template <int WH>
+struct __align__(16) UnitSmem {
+    static constexpr int kRows = kRoiRows + WH - 1;  // source rows of a unit
+    uint4 rows[kRows * kUnitPieces];
+    uint2 codes[8 * kStageStride];                   // codes of eight rows on their way out
+    int need_row[2][kRows];                          // source rows read, in order: this unit's, the next one's
+    int row_of[kRoiRows];                            // marked rows
+};
+
+// A unit: marked rows y0 + i (i in mask) of columns x0 .. x0 + 127 (x0 a multiple of 32)
+// of a plane.
+struct Unit {
+    uint32_t mask;
+    int x0, y0, plane;
+};
+
+__device__ __forceinline__ Unit unit_at(const uint4 *list, int u)
+{
+    const uint4 e = __ldg(list + u);
+    return Unit{e.x, (int)e.y, (int)e.z, (int)e.w};
+}
+
+// Codes of the listed units first, first + step, ... below n, by one warp.  Workspace
+// planes are 256-byte aligned and their pitch is a multiple of 32 codes, so rows leave by
+// bulk copies (codes between a grid's width and the pitch, which no one reads, as 0).
+// One loop over batches of eight source rows: a batch is sliced while the next one's
+// loads are in flight -- the same unit's, or the first of the next unit, whose latency
+// the current unit's codes then cover.
+template <int WW, int WH>
+__device__ __forceinline__ void census_units(const uint4 *list, const PlaneDesc *planes, int first, int n, int step,
+                                             int sentinel, UnitSmem<WH> &sm)
 {
     constexpr int sy = WH / 2;
-    const unsigned full = 0xffffffffu;
-    const int x = x0 + 4 * hl;
-    const bool active = ok && y - sy >= 0 && y + sy < d.Hs;
-    // one load scheme for the whole warp where possible (a uniform branch, so
-    // the other schemes are not executed predicated off): straight word loads
-    // when every lane's twelve pixels lie inside the row; else, at image
-    // borders, word loads where a word lies inside, 0 where it lies outside (it
-    // only feeds pixels whose codes are zeroed) and bytes where it straddles the
-    // end of a row whose width is not a multiple of the word
-    const bool inside = d.vec_load && x >= 4 && (d.k == 1 ? x + 8 <= d.W : 2 * x + 16 <= d.W);
-    uint32_t rows[WH][3];
-    if (__all_sync(full, !active || (inside && d.k == 1))) {
-        if (active) {
-            const uint8_t *p = d.img + (long long)(y - sy) * d.pitch + (x - 4);
+    static_assert(UnitSmem<WH>::kRows <= 32, "a lane per source row");
+    const int lane = threadIdx.x & 31, j = lane & 3, slot = lane >> 2;
+    const uint32_t lt = (1u << lane) - 1u;
+    const Unit none{0u, 0, 0, 0};
+    Unit cur = none, ld = none;                          // the unit being sliced, the unit being loaded
+    Unit nxt = first < n ? unit_at(list, first) : none;
+    int u = first - step;                                // index of `ld`
+    int t = 0, n_need = 0;                               // batch being sliced, source rows of `cur`
+    int tl = 0, nl = 0, bl = 0;                          // batch being loaded, source rows of `ld`
+    PlaneDesc d{};                                       // of `ld`
+    bool vec = false;
+    RowPx px;                                            // the batch being sliced
+    int r = 0;
+    bool on = false;
 #pragma unroll
-            for (int r = 0; r < WH; ++r) {
-                const uint32_t *q = reinterpret_cast<const uint32_t *>(p + (long long)r * d.pitch);
-                rows[r][0] = __ldg(q);
-                rows[r][1] = __ldg(q + 1);
-                rows[r][2] = __ldg(q + 2);
+    for (int i = 0; i < 16; ++i) px.v[i] = 0u;
+    px.left = px.right = 0u;
+    px.pairs = false;
+#pragma unroll 1
+    for (;;) {
+        // the batch after this one
+        if (8 * (tl + 1) < nl) {
+            ++tl;
+        } else {
+            u += step;
+            ld = u < n ? nxt : none;
+            if (u + step < n) nxt = unit_at(list, u + step);
+            tl = 0;
+            bl ^= 1;
+            if (ld.mask) {
+                d = planes[ld.plane];
+                vec = ((reinterpret_cast<uintptr_t>(d.img) | (unsigned)d.pitch) & 15u) == 0;
             }
-        }
-    } else if (__all_sync(full, !active || (inside && d.k == 2))) {
-        if (active) {
-            const uint8_t *p = d.img + 2LL * (y - sy) * d.pitch + 2 * (x - 4);
+            uint32_t need = 0u;  // bit i: source row y0 - sy + i is read
 #pragma unroll
-            for (int r = 0; r < WH; ++r) {
-                const uint2 *q = reinterpret_cast<const uint2 *>(p + 2LL * r * d.pitch);
-                const uint2 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
-                rows[r][0] = __byte_perm(a.x, a.y, 0x6420);
-                rows[r][1] = __byte_perm(b.x, b.y, 0x6420);
-                rows[r][2] = __byte_perm(c.x, c.y, 0x6420);
+            for (int i = 0; i < WH; ++i) need |= ld.mask << i;
+            nl = __popc(need);
+            if ((need >> lane) & 1u) {
+                sm.need_row[bl][__popc(need & lt)] = lane;
+                // the later batches' rows on their way to the L2 while the first is loaded
+                const int yr = ld.y0 - sy + lane;
+                if (yr >= 0 && yr < d.Hs) {
+                    const uint8_t *p = d.img + (long long)d.k * yr * d.pitch;
+                    for (int o = 0; o < kUnitPx * d.k; o += 128)
+                        if (d.k * ld.x0 + o < d.W)
+                            asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p + d.k * ld.x0 + o));
+                }
             }
+            __syncwarp();
         }
-    } else if (__all_sync(full, !active || (d.vec_load && d.k == 1))) {
-        if (active) {
-            const uint8_t *p = d.img + (long long)(y - sy) * d.pitch;
-#pragma unroll
-            for (int r = 0; r < WH; ++r)
-#pragma unroll
-                for (int q = 0; q < 3; ++q) rows[r][q] = word_k1(p + (long long)r * d.pitch, x - 4 + 4 * q, d.W);
+        RowPx px2;
+        const int q = 8 * tl + slot, r2 = q < nl ? sm.need_row[bl][q] : 0, yr = ld.y0 - sy + r2;
+        const bool on2 = q < nl && yr >= 0 && yr < d.Hs;
+        load_row(d, ld.x0, yr, on2, j, vec, px2);
+        if (n_need > 0) slice_row(px, on, j, sm.rows + r * kUnitPieces);
+        px = px2;
+        r = r2;
+        on = on2;
+        if (8 * (t + 1) < n_need) {
+            ++t;
+            continue;
         }
-    } else if (__all_sync(full, !active || (d.vec_load && d.k == 2))) {
-        if (active) {
-            const uint8_t *p = d.img + 2LL * (y - sy) * d.pitch;
-#pragma unroll
-            for (int r = 0; r < WH; ++r)
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    rows[r][q] = word_k2(p + 2LL * r * d.pitch, x - 4 + 4 * q, d.W, d.Ws);
+        if (cur.mask) {  // every source row is sliced: the codes
+            const int n_rows = __popc(cur.mask);
+            if ((cur.mask >> lane) & 1u) sm.row_of[slot_of_row(cur.mask, lane)] = lane;
+            __syncwarp();
+            const PlaneDesc c_d = planes[cur.plane];
+            const int cols = min(kUnitPx, c_d.opitch - cur.x0);
+#pragma unroll 1
+            for (int q0 = 0; q0 < n_rows; q0 += 8) {
+                bulk_wait_read();  // the codes staged before have been read
+                __syncwarp();
+                if (q0 + slot < n_rows) {
+                    uint32_t lo[32], hi[32];
+                    const int i = sm.row_of[q0 + slot];
+                    word_codes<WW, WH>(c_d, cur.x0, cur.y0 + i, j, sm.rows + i * kUnitPieces, sentinel, lo, hi);
+                    stage_codes(sm.codes + slot * kStageStride + j, lo, hi);
+                }
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                __syncwarp();
+                if (lane < 8 && q0 + lane < n_rows)
+                    bulk_row(c_d.out + (long long)(cur.y0 + sm.row_of[q0 + lane]) * c_d.opitch + cur.x0,
+                             sm.codes + lane * kStageStride, cols);
+            }
+            __syncwarp();  // the unit's rows have been read
         }
-    } else if (active) {
-#pragma unroll
-        for (int r = 0; r < WH; ++r) load_row12(d, inside, x, y - sy + r, rows[r]);
+        if (!ld.mask) break;
+        cur = ld;
+        t = 0;
+        n_need = nl;
     }
-    uint64_t c[4] = {0ull, 0ull, 0ull, 0ull};
-    if (active) {
-        auto row = [&](int j, uint32_t (&v)[3]) { v[0] = rows[j][0]; v[1] = rows[j][1]; v[2] = rows[j][2]; };
-        if constexpr (F16)
-            codes4_h<WW, WH>(row, sentinel, c);
-        else
-            codes4<WW, WH>(row, sentinel, c);
-    }
-    if (ok) store4<WW>(d, x, y, active, c);
+    bulk_wait();
 }
 
-__device__ __forceinline__ PlaneDesc desc_of(const Plane &pl)
+inline PlaneDesc desc_of(const Plane &pl)
 {
     PlaneDesc d;
     d.img = pl.img;
     d.out = pl.out;
     d.W = pl.W;
+    d.H = pl.H;
     d.pitch = pl.pitch;
     d.k = pl.k;
     d.Ws = pl.Ws;
     d.Hs = pl.Hs;
     d.opitch = (int)pl.opitch;
     d.vec_load = pl.vec_load;
-    d.pad = 0;
     return d;
 }
 
-// Full image, fixed window: half-warp h of CTA (bx, by) takes tile bx of row by * 16 + h.
+// Full image, fixed window: warp w of CTA (bx, by) takes columns 128 bx .. + 127 of the
+// eight rows 8 (4 by + w) ..; a unit a warp, its codes staged where its rows were.
+template <int WH>
+union __align__(16) FullSmem {
+    uint4 rows[(8 + WH - 1) * kUnitPieces];
+    uint2 codes[8 * kStageStride];
+};
+
 template <int WW, int WH>
-__global__ void __launch_bounds__(256) census_full4_kernel(Plane pl, int sentinel)
+__global__ void __launch_bounds__(kFullThreads, kFullCtas) census_full_unit_kernel(PlaneDesc d, int sentinel)
 {
-    const int y = blockIdx.y * 16 + (threadIdx.x >> 4);
-    // every lane reaches census4 (its load scheme is chosen warp-wide)
-    census4<WW, WH>(desc_of(pl), blockIdx.x * kTile, y, threadIdx.x & 15, y < pl.Hs, sentinel);
+    __shared__ FullSmem<WH> smem[kFullThreads / 32];
+    constexpr int sy = WH / 2;
+    const int lane = threadIdx.x & 31, j = lane & 3, slot = lane >> 2, warp = threadIdx.x >> 5;
+    FullSmem<WH> &sm = smem[warp];
+    const int x0 = blockIdx.x * kUnitPx, y0 = 8 * (blockIdx.y * (kFullThreads / 32) + warp);
+    if (y0 >= d.Hs) return;
+    const bool vec = ((reinterpret_cast<uintptr_t>(d.img) | (unsigned)d.pitch) & 15u) == 0;
+#pragma unroll 1
+    for (int r0 = 0; r0 < 8 + WH - 1; r0 += 8) {
+        const int r = r0 + slot, yr = y0 - sy + r;
+        const bool on = r < 8 + WH - 1 && yr >= 0 && yr < d.Hs;
+        RowPx px;
+        load_row(d, x0, yr, on, j, vec, px);
+        slice_row(px, on, j, sm.rows + (on ? r * kUnitPieces : 0));
+    }
+    __syncwarp();
+    uint32_t lo[32], hi[32];
+    const int rows = min(8, d.Hs - y0), cols = min(kUnitPx, d.Ws - x0);
+    if (slot < rows) word_codes<WW, WH>(d, x0, y0 + slot, j, sm.rows + slot * kUnitPieces, sentinel, lo, hi);
+    __syncwarp();  // the rows have been read
+    if (slot < rows) stage_codes(sm.codes + slot * kStageStride + j, lo, hi);
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    __syncwarp();
+    uint64_t *out = d.out + (long long)y0 * d.opitch + x0;
+    if (((reinterpret_cast<uintptr_t>(d.out) & 15u) | (unsigned)(d.opitch & 1) | (unsigned)(cols & 1)) == 0) {
+        if (lane < rows) bulk_row(out + (long long)lane * d.opitch, sm.codes + lane * kStageStride, cols);
+        bulk_wait();
+    } else {
+        for (int i = 0; i < rows; ++i) {
+            uint2 *dst = reinterpret_cast<uint2 *>(out + (long long)i * d.opitch);
+            for (int c = lane; c < cols; c += 32) dst[c] = sm.codes[i * kStageStride + c];
+        }
+    }
 }
 
 // One 64-pixel tile of row y starting at x0 (x0 a multiple of 64).
-template <int WW, int WH>
-__device__ void census_tile(const Plane &pl, int x0, int y, int win_w, int win_h, int sentinel,
-                            const WarpStage &st)
+__device__ __forceinline__ void census_tile(const Plane &pl, int x0, int y, int win_w, int win_h, int sentinel,
+                                            const WarpStage &st)
 {
     const int lane = threadIdx.x & 31;
     const int sx = win_w / 2, sy = win_h / 2;
@@ -568,34 +635,14 @@ __device__ void census_tile(const Plane &pl, int x0, int y, int win_w, int win_h
         store_pair(pl, x, y, 0ull, 0ull);
         return;
     }
-    uint64_t c0, c1;
-    if constexpr (WW > 0) {
-        stage_rows<WH>(pl, x0, y, st, lane);
-        __syncwarp();
-        tile_codes<WW, WH>(st, lane, sentinel, c0, c1);
-    } else {
-        stage_rows_any(pl, x0, y, sy, st, lane);
-        __syncwarp();
-        c0 = code_any(st, 2 * lane, win_w, win_h, sentinel);
-        c1 = code_any(st, 2 * lane + 1, win_w, win_h, sentinel);
-    }
+    stage_rows_any(pl, x0, y, sy, st, lane);
+    __syncwarp();
+    uint64_t c0 = code_any(st, 2 * lane, win_w, win_h, sentinel);
+    uint64_t c1 = code_any(st, 2 * lane + 1, win_w, win_h, sentinel);
     if (x - sx < 0 || x + sx >= pl.Ws) c0 = 0ull;
     if (x + 1 - sx < 0 || x + 1 + sx >= pl.Ws) c1 = 0ull;
     store_pair(pl, x, y, c0, c1);
     __syncwarp();
-}
-
-__device__ __forceinline__ void census_tile_any(const Plane &pl, int x0, int y, int win_w, int win_h,
-                                                int sentinel, const WarpStage &st)
-{
-    if (win_w == 9 && win_h == 7)
-        census_tile<9, 7>(pl, x0, y, win_w, win_h, sentinel, st);
-    else if (win_w == 7 && win_h == 7)
-        census_tile<7, 7>(pl, x0, y, win_w, win_h, sentinel, st);
-    else if (win_w == 5 && win_h == 5)
-        census_tile<5, 5>(pl, x0, y, win_w, win_h, sentinel, st);
-    else
-        census_tile<0, 0>(pl, x0, y, win_w, win_h, sentinel, st);
 }
 
 // Full image: warp w of CTA (bx, by) takes tile bx of row by * 8 + w.
@@ -607,7 +654,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) census_full_kernel(Plane pl
     const int y = blockIdx.y * kWarpsPerCta + warp;
     if (y >= pl.Hs) return;
     const WarpStage st = warp_stage(stage_mem, warp, win_h);
-    census_tile_any(pl, blockIdx.x * kTile, y, win_w, win_h, sentinel, st);
+    census_tile(pl, blockIdx.x * kTile, y, win_w, win_h, sentinel, st);
 }
 
 // Region of interest.  The planner marks, per plane row, the 32-pixel tiles the
@@ -683,27 +730,89 @@ __global__ void __launch_bounds__(256) tile_list_kernel(MatchArgs a)
     }
 }
 
-// Fixed windows: warp w takes list entries kPer p .. kPer p + kPer - 1 (p = w,
-// w + warps, ...), one per group of kLanes lanes, so all groups run the same
-// instructions in lockstep.  MODE: 0 = 4 CTAs per SM (64 registers),
-// otherwise 3 CTAs per SM.
-template <int WW, int WH, int MODE>
-__global__ void __launch_bounds__(256, MODE == 1 ? 3 : 4) census_roi4_kernel(MatchArgs a)
+// Fixed windows: the units with marked tiles, 16 bytes each in the tile list's place (a
+// bitmap word's 32 rows make at most 16): marked rows of the unit, its first column and
+// row, frame * 4 + plane.  A warp takes 32 rows of one bitmap word column, a row per lane.
+static_assert(2 * kRoiRows == 32, "two units a bitmap word and 32 rows");
+
+struct BandShape {
+    int off[5];  // first (32-row band, word column) item of each plane in a frame, and their number
+};
+
+__global__ void __launch_bounds__(256) unit_list_kernel(MatchArgs a, BandShape bands)
 {
-    constexpr int kLanes = kCensusTilePx / 4;  // lanes per tile (4 pixels each)
-    constexpr int kPer = 32 / kLanes;          // tiles per warp step
-    const int lane = threadIdx.x & 31, hl = lane % kLanes;
-    const int n = a.ws.counts->n_tiles;
-    const int nsteps = (n + kPer - 1) / kPer;
-    const int nw = gridDim.x * (blockDim.x >> 5);
-    const int sentinel = a.p.sentinel;
-    for (int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); p < nsteps; p += nw) {
-        const int t = kPer * p + lane / kLanes;
-        PlaneDesc d;
-        int x0, y;
-        const bool ok = tile_of(a, a.ws.tiles[t < n ? t : kPer * p], d, x0, y) && t < n;
-        census4<WW, WH, MODE == 2>(d, x0, y, hl, ok, sentinel);
+    __shared__ int warp_units[8], warp_tiles[8];
+    __shared__ int s_base;
+    const unsigned full = 0xffffffffu;
+    const long long total = (long long)a.ws.counts->n_frames * bands.off[4];  // clamped by the planner
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long item = (long long)blockIdx.x * 8 + warp;
+    if ((long long)blockIdx.x * 8 >= total) return;  // uniform per CTA
+    uint32_t mine = 0u;  // lane 16 h + u: marked rows of unit u of the h-th half of the rows
+    int col = 0;         // and its first tile of the word
+    int tiles = 0, f = 0, q = 0, band = 0, wi = 0;
+    if (item < total) {
+        f = (int)(item / bands.off[4]);
+        int r = (int)(item - (long long)f * bands.off[4]);
+        while (q < 3 && r >= bands.off[q + 1]) ++q;
+        r -= bands.off[q];
+        const int words = a.ws.bm_row_words[q], rows = (a.ws.bm_plane_off[q + 1] - a.ws.bm_plane_off[q]) / words;
+        band = r / words;
+        wi = r - band * words;
+        const int y = band * 32 + lane;
+        uint32_t bits = 0u;
+        if (y < rows) {
+            uint32_t *p = a.ws.bitmap + f * a.ws.bm_frame_words + a.ws.bm_plane_off[q] + (long long)y * words + wi;
+            bits = *p;
+            if (bits) *p = 0u;  // consumed: clear for the next call
+        }
+        tiles = __reduce_add_sync(full, __popc(bits));
+        // per half of the rows, units from the first marked column not covered yet
+        const unsigned half = lane < kRoiRows ? 0x0000ffffu : 0xffff0000u;
+        uint32_t left = __reduce_or_sync(half, bits);
+        for (int u = 0; __any_sync(full, left != 0u); ++u) {  // at most 8: each takes four columns
+            const int c = left ? __ffs(left) - 1 : 0;
+            const uint32_t m = __ballot_sync(full, left && ((bits >> c) & 15u) != 0u) & half;
+            if ((lane & 15) == u) {
+                mine = lane < kRoiRows ? m : m >> kRoiRows;
+                col = c;
+            }
+            left &= ~(15u << c);
+        }
     }
+    const unsigned found = __ballot_sync(full, mine != 0u);
+    if (lane == 0) {
+        warp_units[warp] = __popc(found);
+        warp_tiles[warp] = tiles;
+    }
+    __syncthreads();
+    int pre = 0, tot = 0, ttot = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        pre += i < warp ? warp_units[i] : 0;
+        tot += warp_units[i];
+        ttot += warp_tiles[i];
+    }
+    if (tot == 0) return;  // uniform per CTA
+    if (threadIdx.x == 0) {
+        s_base = atomicAdd(&a.ws.counts->n_units, tot);
+        atomicAdd(&a.ws.counts->n_tiles, ttot);
+    }
+    __syncthreads();
+    if (mine != 0u)
+        reinterpret_cast<uint4 *>(a.ws.tiles)[s_base + pre + __popc(found & ((1u << lane) - 1u))] =
+            make_uint4(mine, (unsigned)((wi * 32 + col) * kCensusTilePx),
+                       (unsigned)(band * 32 + (lane & kRoiRows)), (unsigned)(f * 4 + q));
+}
+
+template <int WW, int WH>
+__global__ void __launch_bounds__(kUnitThreads, kUnitCtas) census_unit_kernel(MatchArgs a)
+{
+    __shared__ UnitSmem<WH> sm[kUnitThreads / 32];
+    const int warp = threadIdx.x >> 5;
+    census_units<WW, WH>(reinterpret_cast<const uint4 *>(a.ws.tiles), a.ws.planes,
+                         (int)(blockIdx.x + gridDim.x * warp), a.ws.counts->n_units,
+                         (int)gridDim.x * (kUnitThreads / 32), a.p.sentinel, sm[warp]);
 }
 
 // Any other window: a warp per listed tile, rows staged in shared memory.
@@ -730,7 +839,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) census_roi_kernel(MatchArgs
         pl.opitch = d.opitch;
         pl.vec_ok = 1;  // workspace planes: 256-byte aligned, pitch a multiple of 32
         pl.vec_load = d.vec_load;
-        census_tile<0, 0>(pl, x0, y, a.p.win_w, a.p.win_h, a.p.sentinel, st);
+        census_tile(pl, x0, y, a.p.win_w, a.p.win_h, a.p.sentinel, st);
     }
 }
 
@@ -768,13 +877,13 @@ cudaError_t launch_census_single(const uint8_t *img, int W, int H, int pitch, in
     pl.opitch = out_pitch;
     pl.vec_ok = (out_pitch % 2 == 0) && ((reinterpret_cast<uintptr_t>(out) & 15u) == 0);
     pl.vec_load = (k == 1 || k == 2) && (pitch % 4 == 0) && ((reinterpret_cast<uintptr_t>(img) & 7u) == 0);
-    const dim3 grid4(ceil_div_nn(pl.Ws, kTile), ceil_div_nn(pl.Hs, 16));
+    const dim3 units(ceil_div_nn(pl.Ws, kUnitPx), ceil_div_nn(pl.Hs, 8 * (kFullThreads / 32)));
     if (win_w == 9 && win_h == 7) {
-        census_full4_kernel<9, 7><<<grid4, 256, 0, s>>>(pl, sentinel);
+        census_full_unit_kernel<9, 7><<<units, kFullThreads, 0, s>>>(desc_of(pl), sentinel);
     } else if (win_w == 7 && win_h == 7) {
-        census_full4_kernel<7, 7><<<grid4, 256, 0, s>>>(pl, sentinel);
+        census_full_unit_kernel<7, 7><<<units, kFullThreads, 0, s>>>(desc_of(pl), sentinel);
     } else if (win_w == 5 && win_h == 5) {
-        census_full4_kernel<5, 5><<<grid4, 256, 0, s>>>(pl, sentinel);
+        census_full_unit_kernel<5, 5><<<units, kFullThreads, 0, s>>>(desc_of(pl), sentinel);
     } else {
         dim3 grid(ceil_div_nn(pl.Ws, kTile), ceil_div_nn(pl.Hs, kWarpsPerCta));
         census_full_kernel<<<grid, 32 * kWarpsPerCta, census_smem_bytes(win_h), s>>>(pl, win_w, win_h, sentinel);
@@ -782,54 +891,44 @@ cudaError_t launch_census_single(const uint8_t *img, int W, int H, int pitch, in
     return cudaGetLastError();
 }
 
-template <int WW, int WH>
-static int roi4_ctas(int mode)
+int census_roi_ctas_per_sm(int win_w, int win_h)
 {
-    static const int n0 = resident_ctas(census_roi4_kernel<WW, WH, 0>, 256, 0);
-    static const int n1 = resident_ctas(census_roi4_kernel<WW, WH, 1>, 256, 0);
-    static const int n2 = resident_ctas(census_roi4_kernel<WW, WH, 2>, 256, 0);
-    return mode == 0 ? n0 : (mode == 1 ? n1 : n2);
-}
-
-int census_roi_ctas_per_sm(int win_w, int win_h, int mode)
-{
-    if (win_w == 9 && win_h == 7) return roi4_ctas<9, 7>(mode);
-    if (win_w == 7 && win_h == 7) return roi4_ctas<7, 7>(mode);
-    if (win_w == 5 && win_h == 5) return roi4_ctas<5, 5>(mode);
+    static const int n97 = resident_ctas(census_unit_kernel<9, 7>, kUnitThreads, 0);
+    static const int n77 = resident_ctas(census_unit_kernel<7, 7>, kUnitThreads, 0);
+    static const int n55 = resident_ctas(census_unit_kernel<5, 5>, kUnitThreads, 0);
     static const int ng = resident_ctas(census_roi_kernel, 32 * kWarpsPerCta, census_smem_bytes(kMaxWin));
-    return ng;
-}
-
-template <int WW, int WH>
-static void launch_roi4(const MatchArgs &a, int grid, cudaStream_t s)
-{
-    if (a.census_mode == 0)
-        census_roi4_kernel<WW, WH, 0><<<grid, 256, 0, s>>>(a);
-    else if (a.census_mode == 1)
-        census_roi4_kernel<WW, WH, 1><<<grid, 256, 0, s>>>(a);
-    else
-        census_roi4_kernel<WW, WH, 2><<<grid, 256, 0, s>>>(a);
+    if (!census_fixed_window(win_w, win_h)) return ng;
+    return win_h == 5 ? n55 : (win_w == 9 ? n97 : n77);
 }
 
 cudaError_t launch_census_roi(const MatchArgs &a, int sm_count, cudaStream_t s)
 {
-    const long long words = (long long)a.caps.max_frames * a.ws.bm_frame_words;
-    const int list_grid = (int)((words + 255) / 256);
-    if (list_grid > 0) tile_list_kernel<<<list_grid, 256, 0, s>>>(a);
     const int ww = a.p.win_w, wh = a.p.win_h;
-    const int grid = sm_count * census_roi_ctas_per_sm(ww, wh, a.census_mode);
-    // the fixed windows' kernel reads grid columns [x0 - 4, x0 + 36) of a tile, the
-    // generic one [x0 - 8, x0 + 76): census_reach_left/right, which the mapped
+    const int grid = sm_count * census_roi_ctas_per_sm(ww, wh);
+    // a marked tile's codes read grid columns [x0 - 4, x0 + 36) with the fixed windows,
+    // [x0 - 8, x0 + 76) with the generic kernel: census_reach_left/right, which the mapped
     // entry point's gather copies, follow census_fixed_window's choice made here
     if (!census_fixed_window(ww, wh)) {
+        const long long words = (long long)a.caps.max_frames * a.ws.bm_frame_words;
+        const int list_grid = (int)((words + 255) / 256);
+        if (list_grid > 0) tile_list_kernel<<<list_grid, 256, 0, s>>>(a);
         census_roi_kernel<<<grid, 32 * kWarpsPerCta, census_smem_bytes(wh), s>>>(a);
-    } else if (ww == 9 && wh == 7) {
-        launch_roi4<9, 7>(a, grid, s);
-    } else if (ww == 7 && wh == 7) {
-        launch_roi4<7, 7>(a, grid, s);
-    } else {
-        launch_roi4<5, 5>(a, grid, s);
+        return cudaGetLastError();
     }
+    BandShape b;
+    b.off[0] = 0;
+    for (int q = 0; q < 4; ++q) {
+        const int words = a.ws.bm_row_words[q], n = a.ws.bm_plane_off[q + 1] - a.ws.bm_plane_off[q];
+        b.off[q + 1] = b.off[q] + (n > 0 ? ceil_div_nn(n / words, 32) * words : 0);
+    }
+    const long long items = (long long)a.caps.max_frames * b.off[4];
+    if (items > 0) unit_list_kernel<<<(unsigned)((items + 7) / 8), 256, 0, s>>>(a, b);
+    if (ww == 9)
+        census_unit_kernel<9, 7><<<grid, kUnitThreads, 0, s>>>(a);
+    else if (ww == 7)
+        census_unit_kernel<7, 7><<<grid, kUnitThreads, 0, s>>>(a);
+    else
+        census_unit_kernel<5, 5><<<grid, kUnitThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -34,7 +34,8 @@ struct Counts {
     unsigned long long evals;
     int n_big;       // searchable blocks queued from the front (large work)
     int n_small;     // searchable blocks queued from the back (small work)
-    int n_tiles;     // census tiles listed for the region-of-interest census
+    int n_tiles;     // census tiles marked for the region-of-interest census
+    int n_units;     // fixed windows: census units listed (census.cu)
     unsigned long long host_bytes;  // image bytes the gather read from host memory (mapped calls)
 };
 
@@ -79,7 +80,7 @@ struct BlockResult {
 struct PlaneDesc {
     const uint8_t *img;  // source image (full resolution)
     uint64_t *out;       // census plane
-    int W, pitch, k;     // source width, row pitch (bytes), decimation
+    int W, H, pitch, k;  // source width and height, row pitch (bytes), decimation
     int Ws, Hs;          // census grid
     int opitch;          // census row pitch (elements)
     int vec_load;        // word loads allowed (k in {1, 2}, aligned base and pitch)
@@ -136,7 +137,6 @@ struct MatchArgs {
     int strip_cols;            // columns of the shared-memory strip
     int sm_count;              // SMs of the device
     int match_mode;            // 0: tensor-core matcher, 1: two-pass pipelined matcher
-    int census_mode;           // region-of-interest census variant (census.cu)
     int strip_rows;            // rows of the shared-memory strip (pts_side * ndy, rounded up to 4)
     int stats_accumulate;      // 1: the aggregation adds the call's counters to the stats record
     const ctm_frame *gather_src;  // mapped calls: device copy of the caller's frame table (host
@@ -197,7 +197,7 @@ cudaError_t launch_census_single(const uint8_t *img, int W, int H, int pitch, in
 // Region-of-interest census over the marked tiles, `ctas_per_sm` resident CTAs
 // per SM (census_roi_ctas_per_sm; the first call queries the occupancy, so make
 // it before any stream capture).
-int census_roi_ctas_per_sm(int win_w, int win_h, int mode);
+int census_roi_ctas_per_sm(int win_w, int win_h);
 cudaError_t launch_census_roi(const MatchArgs &a, int sm_count, cudaStream_t s);
 size_t census_smem_bytes(int win_h);
 

@@ -67,11 +67,7 @@ int setup_device(int dev)
     }
     st.base = static_cast<unsigned char *>(ptr);
     st.sm_count = sms;
-    for (int m = 0; m < 2; ++m) {  // occupancy queries cached here, once per process
-        ctm::census_roi_ctas_per_sm(9, 7, m);
-        ctm::census_roi_ctas_per_sm(7, 7, m);
-        ctm::census_roi_ctas_per_sm(5, 5, m);
-    }
+    ctm::census_roi_ctas_per_sm(9, 7);  // occupancy queries, cached once per process
     st.ready = true;
     return CTM_OK;
 }
@@ -185,11 +181,9 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     a.nc_stride = nd_max * ndy;
     a.strip_cols = strip_cols;
     a.sm_count = ds.sm_count;
-    a.census_mode = 0;
     a.match_mode = 0;
     a.strip_rows = p->pts_side * ndy;
 
-    census_roi_ctas_per_sm(p->win_w, p->win_h, 0);  // this window's occupancy query, cached after the first
     cudaStream_t s = (cudaStream_t)stream;
     // the census demand bitmap, the counters and the block counts must start at
     // zero (a call interrupted on the device may leave them set)

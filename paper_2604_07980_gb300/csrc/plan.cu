@@ -88,6 +88,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(MatchArgs a, int S)
         const int q = tid;
         d.img = (q & 1) ? fr.right : fr.left;
         d.W = fr.width;
+        d.H = fr.height;
         d.pitch = fr.pitch;
         d.k = q < 2 ? 1 : a.p.close_factor;
         d.Ws = ceil_div_nn(fr.width, d.k);
@@ -97,7 +98,6 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(MatchArgs a, int S)
         d.opitch = (int)(q < 2 ? a.ws.pitch1 : a.ws.pitchk);
         d.vec_load = (d.k == 1 || d.k == 2) && (fr.pitch % 4 == 0) &&
                      ((reinterpret_cast<uintptr_t>(d.img) & 7u) == 0);
-        d.pad = 0;
         a.ws.planes[f * 4 + q] = d;
     }
     const int begin = clampi(fr.box_begin, 0, nb_total);
@@ -457,6 +457,7 @@ __global__ void __launch_bounds__(256) aggregate_kernel(MatchArgs a)
             t.n_big += c.n_big;
             t.n_small += c.n_small;
             t.n_tiles += c.n_tiles;
+            t.n_units += c.n_units;
             t.host_bytes += c.host_bytes;
             *a.ws.stats = t;
         } else {
