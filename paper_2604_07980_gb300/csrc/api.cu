@@ -67,11 +67,12 @@ struct ctm_ctx {
     uint8_t *img_dev = nullptr;
     long long img_pitch = 0;
     ctm_box *boxes_dev = nullptr;
-    float *disp_dev = nullptr;
-    float *depth_dev = nullptr;
-    uint8_t *flags_dev = nullptr;
+    // tables of a host call -- counts, frames, boxes, copied together -- and its results
+    // (disparities, depths, flags one behind the other), in device and page-locked memory
+    char *tables_dev = nullptr, *tables_host = nullptr, *results_dev = nullptr, *results_host = nullptr;
     ctm_frame *frames_host_pinned = nullptr;
     int32_t *counts_host_pinned = nullptr;
+    ctm_box *boxes_host_pinned = nullptr;
     ctm_frame *frames_dev2 = nullptr;
     int32_t *counts_dev2 = nullptr;
     cudaStream_t copy_stream = nullptr;         // host-to-device copies of the sub-batches
@@ -476,8 +477,7 @@ void ctm_destroy(ctm_ctx *ctx)
     if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
     if (ctx->dev_mem) cudaFree(ctx->dev_mem);
     if (ctx->img_dev) cudaFree(ctx->img_dev);
-    if (ctx->frames_host_pinned) cudaFreeHost(ctx->frames_host_pinned);
-    if (ctx->counts_host_pinned) cudaFreeHost(ctx->counts_host_pinned);
+    if (ctx->tables_host) cudaFreeHost(ctx->tables_host);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     for (cudaEvent_t ev : ctx->host_ev)
         if (ev) cudaEventDestroy(ev);
@@ -666,72 +666,94 @@ int ctm_match_batch_profiled(ctm_ctx *ctx, const ctm_frame *frames_dev, const in
 }
 
 // Staging of the host entry points (allocated on first use): device images at
-// a pitch of 128 bytes, boxes and outputs, two frame tables (the staging images'
-// and, for mapped calls, the caller's) in device and page-locked memory, per
-// sub-batch counts, a copy stream and its events.
+// a pitch of 128 bytes; per sub-batch counts, two frame tables (the staging images'
+// and, for mapped calls, the caller's) and boxes, in that order; results; the same two
+// blocks in page-locked memory; a copy stream and its events.
+constexpr size_t kTablesFrames = 256;  // offset of the frame tables, after 4 kHostGroups counts
+static_assert(sizeof(int32_t) * 4 * kHostGroups <= kTablesFrames, "counts of the sub-batches");
+
 static int ensure_host_staging(ctm_ctx *ctx)
 {
     if (ctx->img_dev) return CTM_OK;
     ctx->img_pitch = round_up(ctx->caps.max_width, 128);
-    const size_t img_bytes = (size_t)ctx->img_pitch * ctx->caps.max_height * 2 * ctx->caps.max_frames;
-    size_t off = 0;
-    auto take = [&](size_t bytes) { size_t o = off; off = (size_t)round_up(off + bytes, 256); return o; };
-    const size_t o_img = take(img_bytes);
-    const size_t o_boxes = take(sizeof(ctm_box) * (size_t)ctx->caps.max_boxes);
-    const size_t o_disp = take(sizeof(float) * (size_t)ctx->caps.max_boxes);
-    const size_t o_depth = take(sizeof(float) * (size_t)ctx->caps.max_boxes);
-    const size_t o_flags = take((size_t)ctx->caps.max_boxes);
-    const size_t o_frames = take(sizeof(ctm_frame) * 2 * (size_t)ctx->caps.max_frames);
-    const size_t o_counts = take(sizeof(int32_t) * 4 * kHostGroups);
+    const size_t img_bytes = (size_t)round_up((long long)ctx->img_pitch * ctx->caps.max_height * 2 * ctx->caps.max_frames, 256);
+    const size_t o_boxes = kTablesFrames + (size_t)round_up((long long)(sizeof(ctm_frame) * 2 * ctx->caps.max_frames), 256);
+    const size_t tables = (size_t)round_up((long long)(o_boxes + sizeof(ctm_box) * (size_t)ctx->caps.max_boxes), 256);
+    const size_t results = 9 * (size_t)ctx->caps.max_boxes;  // two floats and a byte each
     void *mem = nullptr;
-    if (dev_alloc(&mem, off) != cudaSuccess) { cudaGetLastError(); return CTM_ENOMEM; }
-    bool okh = cudaMallocHost(&ctx->frames_host_pinned, sizeof(ctm_frame) * 2 * ctx->caps.max_frames) == cudaSuccess &&
-               cudaMallocHost(&ctx->counts_host_pinned, sizeof(int32_t) * 4 * kHostGroups) == cudaSuccess &&
+    if (dev_alloc(&mem, img_bytes + tables + results) != cudaSuccess) { cudaGetLastError(); return CTM_ENOMEM; }
+    bool okh = cudaMallocHost(&ctx->tables_host, tables + results) == cudaSuccess &&
                cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) == cudaSuccess;
     for (cudaEvent_t &ev : ctx->host_ev)
         okh = okh && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess;
     if (!okh) {
         cudaFree(mem);
-        if (ctx->frames_host_pinned) cudaFreeHost(ctx->frames_host_pinned);
-        if (ctx->counts_host_pinned) cudaFreeHost(ctx->counts_host_pinned);
+        if (ctx->tables_host) cudaFreeHost(ctx->tables_host);
         if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
         ctx->copy_stream = nullptr;
         for (cudaEvent_t &ev : ctx->host_ev)
             if (ev) { cudaEventDestroy(ev); ev = nullptr; }
-        ctx->frames_host_pinned = nullptr;
-        ctx->counts_host_pinned = nullptr;
+        ctx->tables_host = nullptr;
         cudaGetLastError();
         return CTM_ENOMEM;
     }
     char *b = static_cast<char *>(mem);
-    ctx->img_dev = reinterpret_cast<uint8_t *>(b + o_img);
-    ctx->boxes_dev = reinterpret_cast<ctm_box *>(b + o_boxes);
-    ctx->disp_dev = reinterpret_cast<float *>(b + o_disp);
-    ctx->depth_dev = reinterpret_cast<float *>(b + o_depth);
-    ctx->flags_dev = reinterpret_cast<uint8_t *>(b + o_flags);
-    ctx->frames_dev2 = reinterpret_cast<ctm_frame *>(b + o_frames);
-    ctx->counts_dev2 = reinterpret_cast<int32_t *>(b + o_counts);
+    ctx->img_dev = reinterpret_cast<uint8_t *>(b);
+    ctx->tables_dev = b + img_bytes;
+    ctx->results_dev = ctx->tables_dev + tables;
+    ctx->results_host = ctx->tables_host + tables;
+    ctx->counts_dev2 = reinterpret_cast<int32_t *>(ctx->tables_dev);
+    ctx->frames_dev2 = reinterpret_cast<ctm_frame *>(ctx->tables_dev + kTablesFrames);
+    ctx->boxes_dev = reinterpret_cast<ctm_box *>(ctx->tables_dev + o_boxes);
+    ctx->counts_host_pinned = reinterpret_cast<int32_t *>(ctx->tables_host);
+    ctx->frames_host_pinned = reinterpret_cast<ctm_frame *>(ctx->tables_host + kTablesFrames);
+    ctx->boxes_host_pinned = reinterpret_cast<ctm_box *>(ctx->tables_host + o_boxes);
     return CTM_OK;
 }
 
+// Counts, frames and the call's boxes in one copy (four copies of a few KB each took
+// about 2 us of the host apiece).
+static cudaError_t copy_tables(ctm_ctx *ctx, const ctm_box *boxes_host, int n_boxes, cudaStream_t s)
+{
+    if (n_boxes > 0) memcpy(ctx->boxes_host_pinned, boxes_host, sizeof(ctm_box) * (size_t)n_boxes);
+    const size_t bytes = (size_t)(reinterpret_cast<char *>(ctx->boxes_host_pinned) - ctx->tables_host) +
+                         sizeof(ctm_box) * (size_t)n_boxes;
+    return cudaMemcpyAsync(ctx->tables_dev, ctx->tables_host, bytes, cudaMemcpyHostToDevice, s);
+}
+
+// Where a host call's kernels put their results: n floats, n floats, n bytes.
+struct HostResults {
+    float *disp, *depth;
+    uint8_t *flags;
+};
+
+static HostResults host_results_at(char *base, int n_boxes)
+{
+    float *f = reinterpret_cast<float *>(base);
+    return HostResults{f, f + n_boxes, reinterpret_cast<uint8_t *>(f + 2 * (size_t)n_boxes)};
+}
+
 // The end of a host call, after its kernels are queued on s: outputs and the
-// call's bounded-wait flag back to host memory, then wait for s.
+// call's bounded-wait flag back to host memory, then wait for s.  The outputs come in one
+// copy to page-locked memory; a copy to the caller's pageable arrays waits for the
+// device on its own, three times.
 static int host_results(ctm_ctx *ctx, cudaStream_t s, int n_boxes, float *disp_host, float *depth_host,
                         uint8_t *flags_host)
 {
     cudaError_t e = cudaSuccess;
-    if (n_boxes > 0) {
-        e = cudaMemcpyAsync(disp_host, ctx->disp_dev, sizeof(float) * n_boxes, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(depth_host, ctx->depth_dev, sizeof(float) * n_boxes, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(flags_host, ctx->flags_dev, (size_t)n_boxes, cudaMemcpyDeviceToHost, s);
-    }
+    if (n_boxes > 0)
+        e = cudaMemcpyAsync(ctx->results_host, ctx->results_dev, 9 * (size_t)n_boxes, cudaMemcpyDeviceToHost, s);
     int32_t *err_h = ctx->counts_host_pinned + 4 * kHostGroups - 1;  // a slot no sub-batch uses
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(err_h, &ctx->ws.stats->error, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) { cudaGetLastError(); return CTM_ECUDA; }
+    if (n_boxes > 0) {
+        const HostResults r = host_results_at(ctx->results_host, n_boxes);
+        memcpy(disp_host, r.disp, sizeof(float) * (size_t)n_boxes);
+        memcpy(depth_host, r.depth, sizeof(float) * (size_t)n_boxes);
+        memcpy(flags_host, r.flags, (size_t)n_boxes);
+    }
     return *err_h ? CTM_ETIMEOUT : CTM_OK;
 }
 
@@ -776,7 +798,15 @@ int ctm_match_batch_host(ctm_ctx *ctx, const ctm_frame *frames_host, int n_frame
             chained = false;
     }
     if (chained && frames_host[n_frames - 1].box_begin + frames_host[n_frames - 1].box_count > n_boxes) chained = false;
-    const int groups = chained ? std::min(kHostGroups, n_frames) : 1;
+    // A sub-batch's kernels are a chain of about 60 us however small it is, so a call is
+    // split only where a part's copy is longer than that (32 MB, 160 us at the link's
+    // rate): eight 1920x1200 pairs (37 MB) 456 -> 390 us in one part instead of four, four
+    // 720p pairs 336 -> 214, twelve 422 -> 328; 32 pairs (147 MB) 1069 us in one part, 979
+    // in two, 944 in four.
+    size_t image_bytes = 0;
+    for (int i = 0; i < n_frames; ++i) image_bytes += 2 * (size_t)frames_host[i].width * (size_t)frames_host[i].height;
+    const int parts = (int)std::min<size_t>(kHostGroups, std::max<size_t>(1, image_bytes >> 25));
+    const int groups = chained ? std::min(parts, n_frames) : 1;
 
     const size_t plane = (size_t)ctx->img_pitch * ctx->caps.max_height;
     cudaStream_t cs = ctx->copy_stream;
@@ -812,48 +842,49 @@ int ctm_match_batch_host(ctm_ctx *ctx, const ctm_frame *frames_host, int n_frame
                 e = cudaMemcpy2DAsync(dst, ctx->img_pitch, src, f.pitch, f.width, f.height, cudaMemcpyHostToDevice, cs);
         }
     };
-    if (e == cudaSuccess && n_boxes > 0)
-        e = cudaMemcpyAsync(ctx->boxes_dev, boxes_host, sizeof(ctm_box) * n_boxes, cudaMemcpyHostToDevice, cs);
     const int grid = ctx->sm_count * ctx->ctas_per_sm;
     // Shrinking sub-batches (12, 10, 6, 4 of 32 frames): each sub-batch's kernels stay
     // shorter than the next sub-batch's copy, and the last one, which nothing
-    // hides, is the smallest.  Below 8 frames, equal parts.
+    // hides, is the smallest.  Below two frames a part, equal parts.
     auto bound = [&](int g) -> int {
-        static const int k64ths[kHostGroups + 1] = {0, 24, 44, 56, 64};  // sub-batch bounds in 64ths
-        if (groups < kHostGroups || n_frames < 8) return (int)((long long)g * n_frames / groups);
-        return (int)(((long long)k64ths[g] * n_frames + 32) / 64);
+        static const int k64ths[kHostGroups][kHostGroups + 1] = {  // sub-batch bounds in 64ths
+            {0, 64}, {0, 44, 64}, {0, 30, 50, 64}, {0, 24, 44, 56, 64}};
+        if (n_frames < 2 * groups) return (int)((long long)g * n_frames / groups);
+        return (int)(((long long)k64ths[groups - 1][g] * n_frames + 32) / 64);
     };
+    // every sub-batch's tables ahead of the images
+    for (int g = 0; g < groups; ++g) {
+        const int f0 = bound(g), f1 = bound(g + 1);
+        const int box0 = groups > 1 ? frames_host[f0].box_begin : 0;
+        for (int i = f0; i < f1; ++i) {
+            ctm_frame t = frames_host[i];
+            t.left = ctx->img_dev + plane * (2 * (size_t)i);
+            t.right = t.left + plane;
+            t.pitch = (int32_t)ctx->img_pitch;
+            t.box_begin -= box0;
+            ctx->frames_host_pinned[i] = t;
+        }
+        ctx->counts_host_pinned[4 * g] = f1 - f0;
+        ctx->counts_host_pinned[4 * g + 1] =
+            groups > 1 ? frames_host[f1 - 1].box_begin + frames_host[f1 - 1].box_count - box0 : n_boxes;
+    }
+    if (e == cudaSuccess) e = copy_tables(ctx, boxes_host, n_boxes, cs);
+    const HostResults res = host_results_at(ctx->results_dev, n_boxes);
     for (int g = 0; g < groups && e == cudaSuccess; ++g) {
         const int f0 = bound(g), f1 = bound(g + 1);
         const int box0 = groups > 1 ? frames_host[f0].box_begin : 0;
-        const int nb = groups > 1 ? frames_host[f1 - 1].box_begin + frames_host[f1 - 1].box_count - box0 : n_boxes;
         for (int i = f0; i < f1 && e == cudaSuccess; ++i) {
             const ctm_frame &f = frames_host[i];
             uint8_t *dl = ctx->img_dev + plane * (2 * (size_t)i);
-            uint8_t *dr = dl + plane;
             image(dl, f.left, f);
-            image(dr, f.right, f);
-            ctm_frame t = f;
-            t.left = dl;
-            t.right = dr;
-            t.pitch = (int32_t)ctx->img_pitch;
-            t.box_begin = f.box_begin - box0;
-            ctx->frames_host_pinned[i] = t;
+            image(dl + plane, f.right, f);
         }
         flush();
-        int32_t *cnt = ctx->counts_host_pinned + 4 * g;
-        cnt[0] = f1 - f0;
-        cnt[1] = nb;
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(ctx->frames_dev2 + f0, ctx->frames_host_pinned + f0, sizeof(ctm_frame) * (f1 - f0),
-                                cudaMemcpyHostToDevice, cs);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(ctx->counts_dev2 + 4 * g, cnt, sizeof(int32_t) * 2, cudaMemcpyHostToDevice, cs);
         if (e == cudaSuccess) e = cudaEventRecord(ctx->host_ev[g], cs);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ctx->host_ev[g], 0);
         if (e != cudaSuccess) break;
         MatchArgs a = make_args(ctx, ctx->frames_dev2 + f0, ctx->counts_dev2 + 4 * g, ctx->boxes_dev + box0,
-                                ctx->disp_dev + box0, ctx->depth_dev + box0, ctx->flags_dev + box0, nullptr);
+                                res.disp + box0, res.depth + box0, res.flags + box0, nullptr);
         a.stats_accumulate = g > 0;  // ctm_get_stats then covers the whole call
         if (enqueue_match(ctx, a, f1 - f0, grid, s, false, 0) != CTM_OK) e = cudaErrorLaunchFailure;
     }
@@ -907,17 +938,11 @@ int ctm_match_batch_mapped(ctm_ctx *ctx, const ctm_frame *frames_host, int n_fra
     int32_t *cnt = ctx->counts_host_pinned;
     cnt[0] = n_frames;
     cnt[1] = n_boxes;
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ctx->frames_dev2, stage, sizeof(ctm_frame) * n_frames, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ctx->frames_dev2 + ctx->caps.max_frames, src, sizeof(ctm_frame) * n_frames,
-                            cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess && n_boxes > 0)
-        e = cudaMemcpyAsync(ctx->boxes_dev, boxes_host, sizeof(ctm_box) * n_boxes, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->counts_dev2, cnt, sizeof(int32_t) * 2, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = copy_tables(ctx, boxes_host, n_boxes, s);
     if (e == cudaSuccess) {
-        MatchArgs a = make_args(ctx, ctx->frames_dev2, ctx->counts_dev2, ctx->boxes_dev, ctx->disp_dev,
-                                ctx->depth_dev, ctx->flags_dev, nullptr);
+        const HostResults res = host_results_at(ctx->results_dev, n_boxes);
+        MatchArgs a = make_args(ctx, ctx->frames_dev2, ctx->counts_dev2, ctx->boxes_dev, res.disp, res.depth,
+                                res.flags, nullptr);
         a.gather_src = ctx->frames_dev2 + ctx->caps.max_frames;
         const int grid = ctx->sm_count * ctx->ctas_per_sm;
         if (enqueue_match(ctx, a, n_frames, grid, s, false, 0) != CTM_OK) e = cudaErrorLaunchFailure;
