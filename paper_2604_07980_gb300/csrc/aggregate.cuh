@@ -20,7 +20,7 @@ __device__ __forceinline__ void aggregate_box(const MatchArgs &a, int box, float
 {
     const unsigned full = 0xffffffffu;
     const BoxPlan P = a.ws.plans[box];
-    const int base = a.ws.blk_base[box];
+    const int base = block_base(a, box);
     float d[2];
     int f[2];
 #pragma unroll
@@ -117,7 +117,7 @@ __device__ __forceinline__ void write_block(const MatchArgs &a, int box, int slo
     BlockResult r;
     r.d_full = rec.d_full;
     r.flags = rec.flags;
-    a.ws.blkres[a.ws.blk_base[box] + slot] = r;
+    a.ws.blkres[block_base(a, box) + slot] = r;
     if (a.dbg.blocks) a.dbg.blocks[(long long)box * (a.p.grid_g * a.p.grid_g) + slot] = rec;
 }
 

@@ -1,8 +1,8 @@
 // api.cu -- the C ABI (include/ctm.h): context, workspace and launch sequences.
 //
-// A match call is six launches on one stream (seven with the two-pass
-// matcher): device planning, point sampling with census demand marking, the
-// census tile list, census of the listed tiles (both images, both
+// A match call is five launches on one stream (six with the two-pass
+// matcher): device planning and point sampling with census demand marking, the
+// list of the marked census tiles, their census (both images, both
 // resolutions), the matching kernel, and the per-box aggregation that writes
 // the outputs.  The batch entry point reads its frame and box counts
 // from device memory, so the whole sequence can be captured once into a CUDA
@@ -221,7 +221,6 @@ int enqueue_match(ctm_ctx *ctx, const MatchArgs &a, int frames_grid, int match_g
         ctx->inject_expiry = 0;
     }
     cudaError_t e = launch_plan(b, s);
-    if (e == cudaSuccess) e = launch_sample(b, s);
     if (e == cudaSuccess && b.gather_src) e = launch_gather(b, ctx->sm_count, s);
     if (e == cudaSuccess) e = launch_census_roi(b, ctx->sm_count, s);
     if (!plain) {
@@ -396,9 +395,7 @@ int ctm_create(ctm_ctx **out, const ctm_params *p, int max_frames, int max_width
     auto take = [&](size_t bytes) { size_t o = off; off = (size_t)round_up(off + bytes, 256); return o; };
     const size_t o_census = take(sizeof(uint64_t) * (size_t)frame_stride * max_frames);
     const size_t o_plans = take(sizeof(BoxPlan) * (size_t)max_boxes);
-    const size_t o_occ = take(sizeof(int4) * (size_t)max_boxes * kMaxOcc);
     const size_t o_nblk = take(sizeof(int) * (size_t)max_boxes);
-    const size_t o_base = take(sizeof(int) * (size_t)max_boxes);
     const size_t o_blkres = take(sizeof(BlockResult) * (size_t)ctx->caps.max_blocks);
     const size_t o_tmaps =
         take(max_frames <= kMaxMapFrames ? sizeof(CUtensorMap) * 4 * kBoxClasses * (size_t)max_frames : 0);
@@ -432,9 +429,7 @@ int ctm_create(ctm_ctx **out, const ctm_params *p, int max_frames, int max_width
     ws.pitch1 = pitch1;
     ws.pitchk = pitchk;
     ws.plans = reinterpret_cast<BoxPlan *>(base + o_plans);
-    ws.occ = reinterpret_cast<int4 *>(base + o_occ);
     ws.nblk = reinterpret_cast<int *>(base + o_nblk);
-    ws.blk_base = reinterpret_cast<int *>(base + o_base);
     ws.blkres = reinterpret_cast<BlockResult *>(base + o_blkres);
     ws.tmaps = reinterpret_cast<const CUtensorMap *>(base + o_tmaps);
     ws.geom = reinterpret_cast<BlockGeom *>(base + o_geom);
@@ -652,7 +647,6 @@ int ctm_match_batch_profiled(ctm_ctx *ctx, const ctm_frame *frames_dev, const in
     cudaError_t e = cudaEventRecord(ev[0], s);
     if (e == cudaSuccess) e = launch_plan(a, s);
     if (e == cudaSuccess) e = cudaEventRecord(ev[1], s);
-    if (e == cudaSuccess) e = launch_sample(a, s);
     if (e == cudaSuccess) e = cudaEventRecord(ev[2], s);
     if (e == cudaSuccess) e = launch_census_roi(a, ctx->sm_count, s);
     if (e == cudaSuccess) e = cudaEventRecord(ev[3], s);

@@ -94,10 +94,8 @@ struct Workspace {
     long long planek_elems;    // elements of one decimated plane
     long long pitch1, pitchk;  // row pitch in elements
     BoxPlan *plans;            // [max_boxes]
-    int4 *occ;                 // [max_boxes * kMaxOcc]
     int *nblk;                 // [max_boxes]
-    int *blk_base;             // [max_boxes]
-    BlockGeom *geom;           // [max_blocks] blk_base[box] + slot
+    BlockGeom *geom;           // [max_blocks] block_base(box) + slot
     int *queue;                // [max_blocks] searchable blocks: large from the front, small from the back
     BlockResult *blkres;       // [max_blocks]
     const CUtensorMap *tmaps;  // [max_frames * 4 * kBoxClasses] census planes L1, R1, Lk, Rk as 2-D
@@ -148,6 +146,9 @@ struct MatchArgs {
 };
 
 __host__ __device__ inline int ceil_div_nn(int a, int b) { return (a + b - 1) / b; }
+
+// First block of a box; grid_g^2 slots each.
+__device__ __forceinline__ int block_base(const MatchArgs &a, int box) { return box * a.p.grid_g * a.p.grid_g; }
 
 // Block at position p of the queue (n_big blocks from the front).
 __device__ __forceinline__ int queue_at(const MatchArgs &a, int n_big, int p)
@@ -204,7 +205,6 @@ size_t census_smem_bytes(int win_h);
 // Planning (plan.cu)
 cudaError_t launch_plan(const MatchArgs &a, cudaStream_t s);
 cudaError_t launch_aggregate(const MatchArgs &a, cudaStream_t s);
-cudaError_t launch_sample(const MatchArgs &a, cudaStream_t s);
 
 // Tensor-core matcher (match_tc.cu) over the queue: blocks in progress are held by
 // workers of match_tc_kernel.  match_tc_configure raises the kernel's shared-memory

@@ -126,9 +126,7 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     const size_t o_stats = take(sizeof(Counts));   // offset kStatsOff
     const size_t o_census = take(sizeof(uint64_t) * (size_t)(2 * plane1 + 2 * planek));
     const size_t o_plans = take(sizeof(BoxPlan) * kMaxBoxes);
-    const size_t o_occ = take(sizeof(int4) * (size_t)kMaxBoxes * kMaxOcc);
     const size_t o_nblk = take(sizeof(int) * kMaxBoxes);
-    const size_t o_base = take(sizeof(int) * kMaxBoxes);
     const size_t o_blkres = take(sizeof(BlockResult) * (size_t)caps.max_blocks);
     const size_t o_geom = take(sizeof(BlockGeom) * (size_t)caps.max_blocks);
     const size_t o_queue = take(sizeof(int) * (size_t)caps.max_blocks);
@@ -147,9 +145,7 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     ws.pitch1 = pitch1;
     ws.pitchk = pitchk;
     ws.plans = reinterpret_cast<BoxPlan *>(b + o_plans);
-    ws.occ = reinterpret_cast<int4 *>(b + o_occ);
     ws.nblk = reinterpret_cast<int *>(b + o_nblk);
-    ws.blk_base = reinterpret_cast<int *>(b + o_base);
     ws.blkres = reinterpret_cast<BlockResult *>(b + o_blkres);
     ws.tmaps = nullptr;  // strips load by 1-D bulk copies
     ws.geom = reinterpret_cast<BlockGeom *>(b + o_geom);
@@ -191,7 +187,6 @@ extern "C" int ctm_match_boxes_noalloc(const ctm_params *p, const uint8_t *left_
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.counts, 0, sizeof(Counts), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.nblk, 0, sizeof(int) * kMaxBoxes, s);
     if (e == cudaSuccess) e = launch_plan(a, s);
-    if (e == cudaSuccess) e = launch_sample(a, s);
     if (e == cudaSuccess) e = launch_census_roi(a, ds.sm_count, s);
     if (e == cudaSuccess) e = launch_match_tc(a, s);
     if (e == cudaSuccess) e = launch_aggregate(a, s);

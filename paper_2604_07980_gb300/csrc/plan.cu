@@ -1,19 +1,15 @@
 // plan.cu -- device-side planning of Algorithm 2's per-box steps.
 //
-// plan_kernel (several CTAs per frame, each a slice of the frame's boxes,
-// a warp per box): clip each box to its frame, classify it FAR
-// or CLOSE by its larger side against tau_s (Sec. 4.3.4), map it to its matching
-// grid (full resolution for FAR, the decimated grid for CLOSE), count its
-// blocks, and select its occluders -- overlapping boxes of the same frame with a
-// larger bottom y (Sec. 4.3.5), nearest (largest bottom y) first, at most
-// max_occluders.  Boxes that are empty after clipping get their outputs here.
-// Each slice's blocks get a contiguous range of block indices.
-//
-// sample_kernel (one warp per row of a box's block grid): the blocks' point grids and
-// usable points; blocks with fewer than min_pts usable points are finished here, the
-// others go to the work queue (large work first) and mark the census tiles
-// their search can read.  All counts come from device memory so a captured
-// graph replays with new inputs.
+// plan_kernel (several CTAs per frame, each a slice of the frame's boxes), a warp per
+// box: clip each box to its frame, classify it FAR or CLOSE by its larger side against
+// tau_s (Sec. 4.3.4), map it to its matching grid (full resolution for FAR, the decimated
+// grid for CLOSE), count its blocks, and select its occluders -- overlapping boxes of the
+// same frame with a larger bottom y (Sec. 4.3.5), nearest (largest bottom y) first, at
+// most max_occluders.  Boxes that are empty after clipping get their outputs here.  Then a
+// warp per row of a box's block grid: the blocks' point grids and usable points; blocks
+// with fewer than min_pts usable points are finished here, the others go to the work
+// queue (large work first) and mark the census tiles their search can read.  All counts
+// come from device memory so a captured graph replays with new inputs.
 #include <math.h>
 
 #include <algorithm>
@@ -59,173 +55,13 @@ __device__ __forceinline__ bool overlaps(int4 a, int4 b)
 constexpr int kStageBoxes = 1024;  // boxes of one frame staged in shared memory
 constexpr int kKeyCache = 8;       // occluder keys per lane held in registers
 
-// S CTAs per frame, each a slice of the frame's boxes: clip, classify,
-// map to the matching grid and select the occluders of every box of the slice
-// (the frame's clipped boxes are staged in shared memory for the pairwise
-// test), then the slice's block counts are scanned and one atomic reserves the
-// slice's range of block indices.
-__global__ void __launch_bounds__(kPlanThreads) plan_kernel(MatchArgs a, int S)
-{
-    __shared__ int4 sbox[kStageBoxes];
-    __shared__ int warp_tot[kPlanThreads / 32];
-    __shared__ int s_run, s_base;
-    const int f = blockIdx.x / S, slice = blockIdx.x % S;
-    const int nf = a.frames ? clampi(a.counts_in[0], 0, a.caps.max_frames) : 1;
-    const int nb_total = clampi(a.frames ? a.counts_in[1] : a.n_boxes1, 0, a.caps.max_boxes);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (blockIdx.x == 0 && tid == 0) {
-        a.ws.counts->n_frames = nf;
-        a.ws.counts->n_boxes = nb_total;
-        a.ws.counts->error = 0;  // the previous call's flag stays until here (see aggregate_kernel)
-    }
-    if (f >= nf) return;
-    const ctm_frame fr = a.frames ? a.frames[f] : a.frame1;
-    const bool bad_frame = fr.width < 1 || fr.height < 1 || fr.width > a.caps.max_width ||
-                           fr.height > a.caps.max_height || fr.pitch < fr.width ||
-                           fr.left == nullptr || fr.right == nullptr;
-    if (slice == 0 && tid < 4) {  // census plane descriptors of this frame: L1, R1, Lk, Rk
-        PlaneDesc d;
-        const int q = tid;
-        d.img = (q & 1) ? fr.right : fr.left;
-        d.W = fr.width;
-        d.H = fr.height;
-        d.pitch = fr.pitch;
-        d.k = q < 2 ? 1 : a.p.close_factor;
-        d.Ws = ceil_div_nn(fr.width, d.k);
-        d.Hs = ceil_div_nn(fr.height, d.k);
-        uint64_t *cb = a.ws.census + (long long)f * a.ws.frame_stride;
-        d.out = q < 2 ? cb + q * a.ws.plane1_elems : cb + 2 * a.ws.plane1_elems + (q - 2) * a.ws.planek_elems;
-        d.opitch = (int)(q < 2 ? a.ws.pitch1 : a.ws.pitchk);
-        d.vec_load = (d.k == 1 || d.k == 2) && (fr.pitch % 4 == 0) &&
-                     ((reinterpret_cast<uintptr_t>(d.img) & 7u) == 0);
-        a.ws.planes[f * 4 + q] = d;
-    }
-    const int begin = clampi(fr.box_begin, 0, nb_total);
-    const int end = clampi(fr.box_begin + fr.box_count, begin, nb_total);
-    const int nloc = end - begin;
-    const bool staged = nloc <= kStageBoxes;
-    if (staged)
-        for (int t = tid; t < nloc; t += blockDim.x) sbox[t] = clip_box(a.boxes[begin + t], fr.width, fr.height);
-    __syncthreads();
-    const ctm_params &p = a.p;
-    const int K = p.max_occluders < kMaxOcc ? p.max_occluders : kMaxOcc;
-    // this CTA's slice of the frame's boxes
-    const int per = (nloc + S - 1) / S;
-    const int sb = begin + min(slice * per, nloc), se = begin + min((slice + 1) * per, nloc);
+constexpr int kPlanWarps = kPlanThreads / 32;
 
-    // a warp per box
-    for (int i = sb + warp; i < se; i += kPlanThreads / 32) {
-        const int4 r = staged ? sbox[i - begin] : clip_box(a.boxes[i], fr.width, fr.height);
-        const int w = r.z - r.x, h = r.w - r.y;
-        const int side = w > h ? w : h;
-        const int far = side < p.far_side_px ? 1 : 0;
-        const int k = far ? 1 : p.close_factor;
-        BoxPlan P;
-        P.cx0 = r.x; P.cy0 = r.y; P.cx1 = r.z; P.cy1 = r.w;
-        // decimated pixel x belongs to the box iff its source pixel k x does
-        P.sx0 = ceil_div_nn(r.x, k); P.sx1 = ceil_div_nn(r.z, k);
-        P.sy0 = ceil_div_nn(r.y, k); P.sy1 = ceil_div_nn(r.w, k);
-        P.frame = f;
-        P.far = far;
-        P.k = k;
-        P.g = far ? 1 : p.grid_g;
-        P.dmin = far ? p.far_dmin : p.close_dmin;
-        P.dmax = far ? p.far_dmax : p.close_dmax;
-        P.Ws = ceil_div_nn(fr.width, k);
-        P.Hs = ceil_div_nn(fr.height, k);
-        P.fb = __fmul_rn(fr.f_px, fr.baseline_m);
-        const bool empty = bad_frame || w <= 0 || h <= 0 || P.sx1 <= P.sx0 || P.sy1 <= P.sy0;
-        P.nblk = empty ? 0 : P.g * P.g;
-
-        // occluders: overlap with positive area and strictly larger bottom y; keep
-        // K of them: frontal ones first (frontal_crop > 0), then by largest bottom
-        // y, ties to the lower index.  Key (frontal, bottom y, -index) is unique
-        // per box, so round t takes the largest key below round t-1's: each lane
-        // scans its share of the frame's boxes.
-        // key of box j as an occluder of box i (0: it is not one)
-        auto occ_key = [&](int j) -> unsigned long long {
-            if (j >= end || j == i) return 0ull;
-            const int4 q = staged ? sbox[j - begin] : clip_box(a.boxes[j], fr.width, fr.height);
-            if (!(q.w > r.w) || !overlaps(r, q)) return 0ull;
-            const unsigned front = frontal(q, fr.width, fr.height, p.frontal_crop) ? 0x80000000u : 0u;
-            return ((unsigned long long)(front | (unsigned)q.w) << 32) | (unsigned)(0x7fffffff - (j - begin));
-        };
-        int nocc = 0;
-        if (!empty && K > 0) {
-            // frames of up to 32 * kKeyCache boxes keep every lane's keys in registers,
-            // so a round is a register scan and two warp reductions
-            const bool cached = nloc <= 32 * kKeyCache;
-            unsigned long long kc[kKeyCache];
-#pragma unroll
-            for (int u = 0; u < kKeyCache; ++u) kc[u] = cached ? occ_key(begin + lane + 32 * u) : 0ull;
-            unsigned long long prev = ~0ull;
-            for (; nocc < K; ++nocc) {
-                unsigned long long best = 0ull;
-                if (cached) {
-#pragma unroll
-                    for (int u = 0; u < kKeyCache; ++u)
-                        if (kc[u] < prev && kc[u] > best) best = kc[u];
-                } else {
-                    for (int j = begin + lane; j < end; j += 32) {
-                        const unsigned long long key = occ_key(j);
-                        if (key < prev && key > best) best = key;
-                    }
-                }
-                // warp maximum of the 64-bit keys (two 32-bit reductions)
-                const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32));
-                const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32) == hi ? (unsigned)best : 0u);
-                best = ((unsigned long long)hi << 32) | lo;
-                if (best == 0ull) break;
-                prev = best;
-                if (lane == 0) {
-                    const int j = begin + (0x7fffffff - (int)lo);
-                    a.ws.occ[(long long)i * kMaxOcc + nocc] =
-                        staged ? sbox[j - begin] : clip_box(a.boxes[j], fr.width, fr.height);
-                }
-            }
-        }
-        P.nocc = nocc;
-        if (lane == 0) {
-            a.ws.plans[i] = P;
-            a.ws.nblk[i] = P.nblk;
-            if (P.nblk == 0) {
-                a.disp[i] = __int_as_float(0x7fc00000);
-                a.depth[i] = __int_as_float(0x7fc00000);
-                a.flags[i] = (uint8_t)((far ? CTM_BOX_FAR : 0) | CTM_BOX_EMPTY);
-            }
-        }
-    }
-    __syncthreads();
-
-    // frame-local exclusive scan of the block counts, one reservation per frame
-    if (tid == 0) s_run = 0;
-    __syncthreads();
-    for (int c0 = sb; c0 < se; c0 += blockDim.x) {
-        const int i = c0 + tid;
-        const int v = i < se ? a.ws.nblk[i] : 0;
-        int x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) warp_tot[warp] = x;
-        __syncthreads();
-        int wpre = 0, tot = 0;
-        for (int wi = 0; wi < kPlanThreads / 32; ++wi) {
-            if (wi < warp) wpre += warp_tot[wi];
-            tot += warp_tot[wi];
-        }
-        if (i < se) a.ws.blk_base[i] = s_run + wpre + x - v;  // slice-local for now
-        __syncthreads();
-        if (tid == 0) s_run += tot;
-        __syncthreads();
-    }
-    if (tid == 0) s_base = atomicAdd(&a.ws.counts->n_blocks, s_run);
-    __syncthreads();
-    const int base = s_base;
-    for (int i = sb + tid; i < se; i += blockDim.x) a.ws.blk_base[i] += base;
-}
+// A planned box and its occluders, for the warps that sample its rows.
+struct PlannedBox {
+    BoxPlan P;
+    int4 occ[kMaxOcc];
+};
 
 // Mark the census row tiles of plane q that columns [c0, c1] of row y lie in.
 __device__ __forceinline__ void mark_range(const MatchArgs &a, int f, int q, int y, int c0, int c1,
@@ -274,22 +110,17 @@ __device__ __forceinline__ void mark_blocks(const MatchArgs &a, const BoxPlan &P
     }
 }
 
-// One warp per row of a box's block grid (FAR boxes: one row of one block), a half-warp
+// Row gb of a box's block grid (FAR boxes: one row of one block), by a warp: a half-warp
 // per block.  The row's blocks share the sampled rows, their occluded rows and mostly
 // their census tiles.  Bound by its instructions (the point grids' divisions, the
 // occluders, the records) and the census marks' atomics, of which neighbouring blocks
-// with touching ranges make one set.  A warp per block took 24.5 us on 32 frames of
-// 1920x1200 (18 K blocks) and 36.9 us on 8 of 3840x2160 (38 K); this 15.1 and 22.3 us.
-__global__ void __launch_bounds__(256) sample_kernel(MatchArgs a, int rows_per_box)
+// with touching ranges make one set.
+__device__ __forceinline__ void sample_row(const MatchArgs &a, const PlannedBox &planned, int box, int gb)
 {
     const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wi = blockIdx.x * 8 + warp;
-    const int box = wi / rows_per_box, gb = wi - box * rows_per_box;
-    if (box >= a.ws.counts->n_boxes || a.ws.nblk[box] == 0) return;
-    const BoxPlan P = a.ws.plans[box];
-    if (gb >= P.g) return;
-    const int base = a.ws.blk_base[box] + gb * P.g;
+    const int lane = threadIdx.x & 31;
+    const BoxPlan P = planned.P;
+    const int base = block_base(a, box) + gb * P.g;
     // the sampled rows; rows beyond ny repeat the last one (no point of theirs is usable)
     const int bw = P.sx1 - P.sx0, bh = P.sy1 - P.sy0;
     const int by0 = P.sy0 + div_small(gb * bh, P.g), by1 = P.sy0 + div_small((gb + 1) * bh, P.g);
@@ -301,7 +132,7 @@ __global__ void __launch_bounds__(256) sample_kernel(MatchArgs a, int rows_per_b
     const int sxw = a.p.win_w >> 1, syw = a.p.win_h >> 1;
     const unsigned rowok = __ballot_sync(full, lane < ny && Yl - syw >= 0 && Yl + syw < P.Hs);
     int4 occ = make_int4(0, 0, 0, 0);
-    if (lane < P.nocc) occ = a.ws.occ[(long long)box * kMaxOcc + lane];
+    if (lane < P.nocc) occ = planned.occ[lane];
     unsigned occrows = 0u;
     const int fy = lane < ny ? P.k * Yl : -1;
     for (int q = 0; q < P.nocc; ++q) {
@@ -417,15 +248,165 @@ __global__ void __launch_bounds__(256) sample_kernel(MatchArgs a, int rows_per_b
         a.ws.queue[a.caps.max_blocks - 1 - qs - __popc(small & lt)] = base + lane;
 }
 
-}  // namespace
-
-cudaError_t launch_sample(const MatchArgs &a, cudaStream_t s)
+// S CTAs per frame, each a slice of the frame's boxes.  First a warp plans a box: clip,
+// classify, map to the matching grid, select its occluders (the frame's clipped boxes are
+// staged in shared memory for the pairwise test).  Then the warps take the rows of the
+// planned boxes' block grids.  Block slot s of box i is block i * grid_g^2 + s, so
+// nothing is counted across CTAs.  Bound by latency (one box's occluder rounds, then one
+// row); the sampling was a kernel of its own, a warp per row with plans and occluders
+// through memory: both 13.4 -> 6.8 us on four boxes, 15.8 -> 9.1 on four 720p frames; a
+// 1279x719 frame 47.9 -> 44.9 us a call, four 720p frames 58.1 -> 56.5, eight 4K frames
+// 294.8 -> 291.5.  64 registers a thread: at the 122 it takes freely, two CTAs an SM, the
+// 4K frames lose it again (293.4).
+__global__ void __launch_bounds__(kPlanThreads, 4) plan_kernel(MatchArgs a, int S)
 {
-    const int rows = std::max(a.p.grid_g, 1);
-    sample_kernel<<<ceil_div_nn(a.caps.max_boxes * rows, 8), 256, 0, s>>>(a, rows);
-    return cudaGetLastError();
+    __shared__ int4 sbox[kStageBoxes];
+    __shared__ PlannedBox planned[kPlanWarps];
+    const int f = blockIdx.x / S, slice = blockIdx.x % S;
+    const int nf = a.frames ? clampi(a.counts_in[0], 0, a.caps.max_frames) : 1;
+    const int nb_total = clampi(a.frames ? a.counts_in[1] : a.n_boxes1, 0, a.caps.max_boxes);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (blockIdx.x == 0 && tid == 0) {
+        a.ws.counts->n_frames = nf;
+        a.ws.counts->n_boxes = nb_total;
+        a.ws.counts->error = 0;  // the previous call's flag stays until here (see aggregate_kernel)
+    }
+    if (f >= nf) return;
+    const ctm_frame fr = a.frames ? a.frames[f] : a.frame1;
+    const bool bad_frame = fr.width < 1 || fr.height < 1 || fr.width > a.caps.max_width ||
+                           fr.height > a.caps.max_height || fr.pitch < fr.width ||
+                           fr.left == nullptr || fr.right == nullptr;
+    if (slice == 0 && tid < 4) {  // census plane descriptors of this frame: L1, R1, Lk, Rk
+        PlaneDesc d;
+        const int q = tid;
+        d.img = (q & 1) ? fr.right : fr.left;
+        d.W = fr.width;
+        d.H = fr.height;
+        d.pitch = fr.pitch;
+        d.k = q < 2 ? 1 : a.p.close_factor;
+        d.Ws = ceil_div_nn(fr.width, d.k);
+        d.Hs = ceil_div_nn(fr.height, d.k);
+        uint64_t *cb = a.ws.census + (long long)f * a.ws.frame_stride;
+        d.out = q < 2 ? cb + q * a.ws.plane1_elems : cb + 2 * a.ws.plane1_elems + (q - 2) * a.ws.planek_elems;
+        d.opitch = (int)(q < 2 ? a.ws.pitch1 : a.ws.pitchk);
+        d.vec_load = (d.k == 1 || d.k == 2) && (fr.pitch % 4 == 0) &&
+                     ((reinterpret_cast<uintptr_t>(d.img) & 7u) == 0);
+        a.ws.planes[f * 4 + q] = d;
+    }
+    const int begin = clampi(fr.box_begin, 0, nb_total);
+    const int end = clampi(fr.box_begin + fr.box_count, begin, nb_total);
+    const int nloc = end - begin;
+    const bool staged = nloc <= kStageBoxes;
+    if (staged)
+        for (int t = tid; t < nloc; t += blockDim.x) sbox[t] = clip_box(a.boxes[begin + t], fr.width, fr.height);
+    __syncthreads();
+    const ctm_params &p = a.p;
+    const int K = p.max_occluders < kMaxOcc ? p.max_occluders : kMaxOcc;
+    // this CTA's slice of the frame's boxes, as many at a time as it has warps
+    const int per = (nloc + S - 1) / S;
+    const int sb = begin + min(slice * per, nloc), se = begin + min((slice + 1) * per, nloc);
+
+    for (int i0 = sb; i0 < se; i0 += kPlanWarps) {
+        // a warp per box
+        const int i = i0 + warp;
+        if (i < se) {
+            const int4 r = staged ? sbox[i - begin] : clip_box(a.boxes[i], fr.width, fr.height);
+            const int w = r.z - r.x, h = r.w - r.y;
+            const int side = w > h ? w : h;
+            const int far = side < p.far_side_px ? 1 : 0;
+            const int k = far ? 1 : p.close_factor;
+            BoxPlan P;
+            P.cx0 = r.x; P.cy0 = r.y; P.cx1 = r.z; P.cy1 = r.w;
+            // decimated pixel x belongs to the box iff its source pixel k x does
+            P.sx0 = ceil_div_nn(r.x, k); P.sx1 = ceil_div_nn(r.z, k);
+            P.sy0 = ceil_div_nn(r.y, k); P.sy1 = ceil_div_nn(r.w, k);
+            P.frame = f;
+            P.far = far;
+            P.k = k;
+            P.g = far ? 1 : p.grid_g;
+            P.dmin = far ? p.far_dmin : p.close_dmin;
+            P.dmax = far ? p.far_dmax : p.close_dmax;
+            P.Ws = ceil_div_nn(fr.width, k);
+            P.Hs = ceil_div_nn(fr.height, k);
+            P.fb = __fmul_rn(fr.f_px, fr.baseline_m);
+            const bool empty = bad_frame || w <= 0 || h <= 0 || P.sx1 <= P.sx0 || P.sy1 <= P.sy0;
+            P.nblk = empty ? 0 : P.g * P.g;
+
+            // occluders: overlap with positive area and strictly larger bottom y; keep
+            // K of them: frontal ones first (frontal_crop > 0), then by largest bottom
+            // y, ties to the lower index.  Key (frontal, bottom y, -index) is unique
+            // per box, so round t takes the largest key below round t-1's: each lane
+            // scans its share of the frame's boxes.
+            // key of box j as an occluder of box i (0: it is not one)
+            auto occ_key = [&](int j) -> unsigned long long {
+                if (j >= end || j == i) return 0ull;
+                const int4 q = staged ? sbox[j - begin] : clip_box(a.boxes[j], fr.width, fr.height);
+                if (!(q.w > r.w) || !overlaps(r, q)) return 0ull;
+                const unsigned front = frontal(q, fr.width, fr.height, p.frontal_crop) ? 0x80000000u : 0u;
+                return ((unsigned long long)(front | (unsigned)q.w) << 32) | (unsigned)(0x7fffffff - (j - begin));
+            };
+            int nocc = 0;
+            int4 occ = make_int4(0, 0, 0, 0);  // lane q: occluder q
+            if (!empty && K > 0) {
+                // frames of up to 32 * kKeyCache boxes keep every lane's keys in registers,
+                // so a round is a register scan and two warp reductions
+                const bool cached = nloc <= 32 * kKeyCache;
+                unsigned long long kc[kKeyCache];
+#pragma unroll
+                for (int u = 0; u < kKeyCache; ++u) kc[u] = cached ? occ_key(begin + lane + 32 * u) : 0ull;
+                unsigned long long prev = ~0ull;
+                for (; nocc < K; ++nocc) {
+                    unsigned long long best = 0ull;
+                    if (cached) {
+#pragma unroll
+                        for (int u = 0; u < kKeyCache; ++u)
+                            if (kc[u] < prev && kc[u] > best) best = kc[u];
+                    } else {
+                        for (int j = begin + lane; j < end; j += 32) {
+                            const unsigned long long key = occ_key(j);
+                            if (key < prev && key > best) best = key;
+                        }
+                    }
+                    // warp maximum of the 64-bit keys (two 32-bit reductions)
+                    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32));
+                    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32) == hi ? (unsigned)best : 0u);
+                    best = ((unsigned long long)hi << 32) | lo;
+                    if (best == 0ull) break;
+                    prev = best;
+                    if (lane == nocc) {
+                        const int j = begin + (0x7fffffff - (int)lo);
+                        occ = staged ? sbox[j - begin] : clip_box(a.boxes[j], fr.width, fr.height);
+                    }
+                }
+            }
+            P.nocc = nocc;
+            if (lane == 0) {
+                if (P.nblk == 0) {
+                    a.disp[i] = __int_as_float(0x7fc00000);
+                    a.depth[i] = __int_as_float(0x7fc00000);
+                    a.flags[i] = (uint8_t)((far ? CTM_BOX_FAR : 0) | CTM_BOX_EMPTY);
+                } else if (atomicCAS(a.ws.nblk + i, 0, P.nblk) == 0) {
+                    a.ws.plans[i] = P;
+                    atomicAdd(&a.ws.counts->n_blocks, P.nblk);
+                } else {
+                    P.nblk = 0;  // frames whose boxes overlap: the box is another frame's
+                }
+                planned[warp].P = P;
+            }
+            planned[warp].occ[lane] = occ;
+        }
+        __syncthreads();
+        // a warp per row of their block grids
+        const int rows = a.p.grid_g, n = min(se - i0, kPlanWarps);
+        for (int t = warp; t < n * rows; t += kPlanWarps) {
+            const int q = t / rows, gb = t - q * rows;
+            if (planned[q].P.nblk > 0 && gb < planned[q].P.g) sample_row(a, planned[q], i0 + q, gb);
+        }
+        __syncthreads();
+    }
 }
 
+}  // namespace
 
 // One warp per planned box with blocks: Sec. 4.3.4 over its block records and
 // Eq. 1 (boxes without blocks got their outputs from the planner).
@@ -490,15 +471,14 @@ cudaError_t launch_aggregate(const MatchArgs &a, cudaStream_t s)
 }
 
 // The counters and block counts start at zero: the workspace is created zeroed
-// and every call's aggregate_kernel zeroes them again.  A frame's boxes are
-// planned a warp per box, so a frame with many boxes gets more CTAs when the
-// call has few frames: about two CTAs per SM over the call's frame capacity,
-// at least 4 and at most 32 per frame.
+// and every call's aggregate_kernel zeroes them again.  Two boxes a CTA at the context's
+// capacity (their rows then fill its warps; with four a 1279x719 frame takes 49.3 us, with
+// one 32 frames of 1920x1200 221.8 instead of 218.9), 4 to 64 CTAs per frame.
 cudaError_t launch_plan(const MatchArgs &a, cudaStream_t s)
 {
-    const int nf = a.caps.max_frames > 0 ? a.caps.max_frames : 1;
-    const int slices = std::min(std::max(ceil_div_nn(2 * a.sm_count, nf), 4), 32);
-    plan_kernel<<<a.caps.max_frames * slices, kPlanThreads, 0, s>>>(a, slices);
+    const int nf = std::max(a.caps.max_frames, 1);
+    const int slices = std::min(std::max(ceil_div_nn(a.caps.max_boxes, 2 * nf), 4), 64);
+    plan_kernel<<<nf * slices, kPlanThreads, 0, s>>>(a, slices);
     return cudaGetLastError();
 }
 
