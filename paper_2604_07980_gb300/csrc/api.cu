@@ -243,12 +243,24 @@ void drop_single_graph(ctm_ctx *ctx)
     ctx->sgraph = nullptr;
 }
 
+// While it lives, this thread may make calls (graph instantiation) that a capture in
+// progress on another stream would forbid it, which would end that capture; nothing done
+// here enters it.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Capture the launches of a single-frame call.  They form a chain: the first node
 // (plan_kernel) and the last (aggregate_kernel) are the only ones that read the caller's
 // pointers, so later calls set those two nodes' arguments.  False if it cannot be built.
 bool build_single_graph(ctm_ctx *ctx, const MatchArgs &a, int grid)
 {
-    if (cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return false;
+    if (cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
     const int r = enqueue_match(ctx, a, 1, grid, ctx->capture_stream, false, 0, false);
     cudaError_t e = cudaStreamEndCapture(ctx->capture_stream, &ctx->sgraph);
     bool ok = r == CTM_OK && e == cudaSuccess && ctx->sgraph;
@@ -528,6 +540,7 @@ int ctm_match_boxes(ctm_ctx *ctx, const uint8_t *left_dev, const uint8_t *right_
     // row); not for diagnostics, an armed fault injection or a stream being captured.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     bool replay = ctx->single_calls > 0 && !dbg && !ctx->inject_expiry;
+    RelaxedCapture relaxed;
     if (replay && (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)) {
         cudaGetLastError();
         replay = false;

@@ -63,3 +63,36 @@ def test_replayed_single_frame_calls_equal_oracle():
     torch.cuda.synchronize()
     compare_box_outputs({k: out[k].cpu().numpy() for k in ("disp", "depth", "flags")}, ref, "captured, other boxes")
     ctx.close()
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local", "relaxed"])
+def test_replay_beside_a_capture(mode):
+    """Calls on one stream while the same thread captures another stream: the replay's graph is
+    built and launched, and the caller's capture stays valid, in every capture mode."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2604_07980_gb300 import binding as B
+    w = wl.frame1080(seed=5300, W=640, H=360, n_boxes=9, side_range=(12, 150))
+    f = w.frames[0]
+    L, R = torch_frames(w.frames)[0]
+    b = torch.from_numpy(np.ascontiguousarray(w.boxes)).cuda()
+    ref = orc.match_frame(f.left, f.right, w.boxes, f.f_px, f.baseline_m, orc.Params(**w.params))
+    n = len(w.boxes)
+    outs = [(torch.empty(n, device="cuda"), torch.empty(n, device="cuda"),
+             torch.empty(n, dtype=torch.uint8, device="cuda")) for _ in range(3)]
+    x = torch.zeros(8, device="cuda")
+    ctx = B.Context(w.params, 1, 640, 360, 16)
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, capture_error_mode=mode):
+        x.add_(1)
+        for out in outs:
+            ctx.match_boxes(L, R, b, f.f_px, f.baseline_m, out=out, stream=side)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert (x == 1).all()
+    for i, out in enumerate(outs):
+        got = {k: v.cpu().numpy() for k, v in zip(("disp", "depth", "flags"), out)}
+        compare_box_outputs(got, ref, f"beside a {mode} capture, call {i}")
+    ctx.close()
