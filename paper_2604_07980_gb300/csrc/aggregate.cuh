@@ -1,5 +1,5 @@
 // aggregate.cuh -- block records and per-box aggregation (Sec. 4.3.4).  The
-// sampling kernel (blocks with too few points) and the matching kernels
+// planner (blocks with too few points) and the matching kernels
 // (searched blocks) write block records; aggregate_kernel (plan.cu) then
 // aggregates every box with one warp.
 #pragma once

@@ -503,8 +503,9 @@ int ctm_census_build(const uint8_t *img_dev, int width, int height, int pitch, i
         return CTM_EINVAL;
     const int Ws = (width + factor - 1) / factor;
     if (codes_pitch < Ws) return CTM_EINVAL;
-    cudaError_t e = launch_census_single(img_dev, width, height, pitch, factor, win_w, win_h,
-                                         sentinel, codes_dev, codes_pitch, (cudaStream_t)stream);
+    const CensusImage image{img_dev, width, height, codes_dev};
+    cudaError_t e = launch_census_images(&image, 1, pitch, factor, win_w, win_h, sentinel, codes_pitch,
+                                         (cudaStream_t)stream);
     return e == cudaSuccess ? CTM_OK : CTM_ECUDA;
 }
 

@@ -586,15 +586,20 @@ union __align__(16) FullSmem {
     uint2 codes[8 * kStageStride];
 };
 
+struct PlanePair {
+    PlaneDesc d[2];
+};
+
 template <int WW, int WH>
-__global__ void __launch_bounds__(kFullThreads, kFullCtas) census_full_unit_kernel(PlaneDesc d, int sentinel)
+__global__ void __launch_bounds__(kFullThreads, kFullCtas) census_full_unit_kernel(PlanePair planes, int sentinel)
 {
+    const PlaneDesc &d = planes.d[blockIdx.z];  // one image, or two in one launch
     __shared__ FullSmem<WH> smem[kFullThreads / 32];
     constexpr int sy = WH / 2;
     const int lane = threadIdx.x & 31, j = lane & 3, slot = lane >> 2, warp = threadIdx.x >> 5;
     FullSmem<WH> &sm = smem[warp];
     const int x0 = blockIdx.x * kUnitPx, y0 = 8 * (blockIdx.y * (kFullThreads / 32) + warp);
-    if (y0 >= d.Hs) return;
+    if (y0 >= d.Hs || x0 >= d.Ws) return;
     const bool vec = ((reinterpret_cast<uintptr_t>(d.img) | (unsigned)d.pitch) & 15u) == 0;
 #pragma unroll 1
     for (int r0 = 0; r0 < 8 + WH - 1; r0 += 8) {
@@ -658,11 +663,10 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) census_full_kernel(Plane pl
 }
 
 // Region of interest.  The planner marks, per plane row, the 32-pixel tiles the
-// search reads (bitmap, one bit per tile).  tile_list_kernel compacts the
-// marks into a dense list (one packed entry per tile, row-major within each
-// 256-word chunk of the bitmap) and clears the bitmap for the next call; the
-// census kernels then take tiles from the list, so every warp gets the same
-// share of work and no warp scans empty bitmap words.
+// search reads (bitmap, one bit per tile).  A list kernel compacts the marks into a
+// dense list -- units for the fixed windows (unit_list_kernel), else tiles, one packed
+// entry each (tile_list_kernel) -- and clears the bitmap for the next call; the census
+// kernels then take their work from the list, so no warp scans empty bitmap words.
 //
 // Entry: bits 0-9 tile (x0 / 32), 10-25 row, 26-27 plane (L1, R1, Lk, Rk), 28- frame.
 __device__ __forceinline__ unsigned long long tile_entry(int f, int q, int y, int tile)
@@ -861,33 +865,45 @@ size_t census_smem_bytes(int win_h)
     return sizeof(uint32_t) * (size_t)kWarpsPerCta * 2 * win_h * kWordsMax;
 }
 
-cudaError_t launch_census_single(const uint8_t *img, int W, int H, int pitch, int k, int win_w,
-                                 int win_h, int sentinel, uint64_t *out, long long out_pitch,
-                                 cudaStream_t s)
+static Plane plane_of(const CensusImage &c, int pitch, int k, long long out_pitch)
 {
     Plane pl;
-    pl.img = img;
-    pl.W = W;
-    pl.H = H;
+    pl.img = c.img;
+    pl.W = c.W;
+    pl.H = c.H;
     pl.pitch = pitch;
     pl.k = k;
-    pl.Ws = ceil_div_nn(W, k);
-    pl.Hs = ceil_div_nn(H, k);
-    pl.out = out;
+    pl.Ws = ceil_div_nn(c.W, k);
+    pl.Hs = ceil_div_nn(c.H, k);
+    pl.out = c.out;
     pl.opitch = out_pitch;
-    pl.vec_ok = (out_pitch % 2 == 0) && ((reinterpret_cast<uintptr_t>(out) & 15u) == 0);
-    pl.vec_load = (k == 1 || k == 2) && (pitch % 4 == 0) && ((reinterpret_cast<uintptr_t>(img) & 7u) == 0);
-    const dim3 units(ceil_div_nn(pl.Ws, kUnitPx), ceil_div_nn(pl.Hs, 8 * (kFullThreads / 32)));
-    if (win_w == 9 && win_h == 7) {
-        census_full_unit_kernel<9, 7><<<units, kFullThreads, 0, s>>>(desc_of(pl), sentinel);
-    } else if (win_w == 7 && win_h == 7) {
-        census_full_unit_kernel<7, 7><<<units, kFullThreads, 0, s>>>(desc_of(pl), sentinel);
-    } else if (win_w == 5 && win_h == 5) {
-        census_full_unit_kernel<5, 5><<<units, kFullThreads, 0, s>>>(desc_of(pl), sentinel);
-    } else {
-        dim3 grid(ceil_div_nn(pl.Ws, kTile), ceil_div_nn(pl.Hs, kWarpsPerCta));
-        census_full_kernel<<<grid, 32 * kWarpsPerCta, census_smem_bytes(win_h), s>>>(pl, win_w, win_h, sentinel);
+    pl.vec_ok = (out_pitch % 2 == 0) && ((reinterpret_cast<uintptr_t>(c.out) & 15u) == 0);
+    pl.vec_load = (k == 1 || k == 2) && (pitch % 4 == 0) && ((reinterpret_cast<uintptr_t>(c.img) & 7u) == 0);
+    return pl;
+}
+
+cudaError_t launch_census_images(const CensusImage *images, int n, int pitch, int k, int win_w, int win_h,
+                                 int sentinel, long long out_pitch, cudaStream_t s)
+{
+    PlanePair pair{};
+    int Ws = 0, Hs = 0;
+    for (int i = 0; i < n; ++i) {
+        const Plane pl = plane_of(images[i], pitch, k, out_pitch);
+        pair.d[i] = desc_of(pl);
+        Ws = pl.Ws > Ws ? pl.Ws : Ws;
+        Hs = pl.Hs > Hs ? pl.Hs : Hs;
+        if (!census_fixed_window(win_w, win_h)) {
+            const dim3 grid(ceil_div_nn(pl.Ws, kTile), ceil_div_nn(pl.Hs, kWarpsPerCta));
+            census_full_kernel<<<grid, 32 * kWarpsPerCta, census_smem_bytes(win_h), s>>>(pl, win_w, win_h, sentinel);
+        }
     }
+    const dim3 units(ceil_div_nn(Ws, kUnitPx), ceil_div_nn(Hs, 8 * (kFullThreads / 32)), n);
+    if (win_w == 9 && win_h == 7)
+        census_full_unit_kernel<9, 7><<<units, kFullThreads, 0, s>>>(pair, sentinel);
+    else if (win_w == 7 && win_h == 7)
+        census_full_unit_kernel<7, 7><<<units, kFullThreads, 0, s>>>(pair, sentinel);
+    else if (win_w == 5 && win_h == 5)
+        census_full_unit_kernel<5, 5><<<units, kFullThreads, 0, s>>>(pair, sentinel);
     return cudaGetLastError();
 }
 

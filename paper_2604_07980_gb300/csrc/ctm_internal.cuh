@@ -18,7 +18,7 @@ constexpr int kMaxOcc = 32;
 constexpr int kMaxWin = 15;
 constexpr int kPlanThreads = 256;
 
-// The sampling kernel queues the searchable blocks in sampling order (boxes of a
+// The planner queues the searchable blocks in sampling order (boxes of a
 // frame together, so blocks whose strips overlap run close in time and share the
 // L2): blocks with at least kBigWork usable points x candidates from the front,
 // the others from the back.
@@ -50,7 +50,7 @@ struct BoxPlan {
 };
 
 // Sampled point grid of one block (Sec. 4.3.4) with its usable points
-// (Sec. 4.3.5), computed once by the sampling kernel.
+// (Sec. 4.3.5), computed once by the planner.
 struct __align__(16) BlockGeom {
     int16_t X[kMaxPtsSide];           // sampled columns on the matching grid
     int16_t Y[kMaxPtsSide];           // sampled rows
@@ -177,9 +177,8 @@ __device__ __forceinline__ int point_coord(int b0, int b1, int n, int j)
 // Census launches (census.cu)
 constexpr int kCensusTilePx = 32;   // pixels per bitmap bit (a census tile: 8 lanes x 4 pixels)
 // Grid columns a census tile x0 .. x0 + 31 reads: [x0 - L, x0 + R).  The fixed
-// windows (5x5, 7x7, 9x7; census_roi4_kernel) load twelve pixels x - 4 .. x + 7
-// per lane of four pixels; the other windows (census_roi_kernel) load 21 words
-// of four pixels from x0 - 8.  Rows: the window's rows around the tile's row.
+// windows (5x5, 7x7, 9x7; census_unit_kernel) reach at most four columns; the
+// other windows (census_roi_kernel) load 21 words of four pixels from x0 - 8.  Rows: the window's rows around the tile's row.
 __host__ __device__ inline bool census_fixed_window(int win_w, int win_h)
 {
     return (win_w == 9 && win_h == 7) || (win_w == 7 && win_h == 7) || (win_w == 5 && win_h == 5);
@@ -187,14 +186,19 @@ __host__ __device__ inline bool census_fixed_window(int win_w, int win_h)
 __host__ __device__ inline int census_reach_left(int win_w, int win_h) { return census_fixed_window(win_w, win_h) ? 4 : 8; }
 __host__ __device__ inline int census_reach_right(int win_w, int win_h) { return census_fixed_window(win_w, win_h) ? 36 : 76; }
 
-// Mapped calls (gather.cu): after the sampling kernel has marked the census
+// Mapped calls (gather.cu): after the planner has marked the census
 // tiles, copy from the caller's host images into the staging images the source
 // bytes those tiles' census reads (64-byte segments of each source row).
 cudaError_t launch_gather(const MatchArgs &a, int sm_count, cudaStream_t s);
 constexpr int kGatherSegBytes = 64;
-cudaError_t launch_census_single(const uint8_t *img, int W, int H, int pitch, int k, int win_w,
-                                 int win_h, int sentinel, uint64_t *out, long long out_pitch,
-                                 cudaStream_t s);
+// Census of one image or two (n) of the same pitches, in one launch for the fixed windows.
+struct CensusImage {
+    const uint8_t *img;
+    int W, H;
+    uint64_t *out;
+};
+cudaError_t launch_census_images(const CensusImage *images, int n, int pitch, int k, int win_w, int win_h,
+                                 int sentinel, long long out_pitch, cudaStream_t s);
 // Region-of-interest census over the marked tiles, `ctas_per_sm` resident CTAs
 // per SM (census_roi_ctas_per_sm; the first call queries the occupancy, so make
 // it before any stream capture).

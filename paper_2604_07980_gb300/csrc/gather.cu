@@ -2,7 +2,7 @@
 // from the caller's host memory (ctm_match_batch_mapped).
 //
 // The planner knows before any pixel moves which census tiles the search will
-// read: the sampling kernel marks them in the demand bitmap (one bit per
+// read: the planner marks them in the demand bitmap (one bit per
 // 32-pixel tile of a plane row).  A tile's census reads a fixed window of its
 // plane (grid columns [x0 - L, x0 + R) of the window's rows; see
 // census_reach_left/right), which at decimation k is every k-th column and row
@@ -11,7 +11,7 @@
 // bitmap whether any marked tile of a plane made from this image reads its
 // segment, then the warp copies the needed segments from host memory into the
 // staging image.  Bytes of the staging images that no marked tile reads are never
-// written and never read.  The bitmap is read, not cleared (tile_list_kernel
+// written and never read.  The bitmap is read, not cleared (the list kernel
 // consumes it next).
 #include <algorithm>
 

@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(NT) match_box_kernel(MatchArgs a, int box)
     __shared__ __align__(16) Shared sh;
     if ((int)blockIdx.x >= a.ws.nblk[box]) return;
     const int b = block_base(a, box) + blockIdx.x;
-    if (a.ws.geom[b].n_valid < a.p.min_pts) return;  // finished by the sampling kernel
+    if (a.ws.geom[b].n_valid < a.p.min_pts) return;  // finished by the planner
     const Smem sm = carve(a, smem_raw);
     if (threadIdx.x < (int)(sizeof(BlockGeom) / 16))
         cp_async16(reinterpret_cast<char *>(&sh.geom) + 16 * threadIdx.x,

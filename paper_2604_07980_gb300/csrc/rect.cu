@@ -77,8 +77,8 @@ __global__ void __launch_bounds__(kRectThreads) rect_kernel(const uint64_t *CL, 
 // its candidates: (n + 2 nd - 2) nd costs instead of 2 n nd, half for a wide segment.
 // Half the population counts (the bound of rect_kernel, at 0.72 of their peak; 0.70 here)
 // for one shuffle, select and minimum more a cost.  A 1920x128 band of a 1920x1200
-// pair, 64 disparities, 9 offsets: the call 0.156 -> 0.102 ms, of which 0.03 ms are the
-// census of the band's rows instead of both whole images.
+// pair, 64 disparities, 9 offsets: the call 0.156 -> 0.100 ms, 0.088 of it this kernel;
+// the census of both images' band rows is one launch of 8 us (0.106 ms with two).
 constexpr int kBandThreads = 256;
 constexpr int kBandGroups = 2;       // 32-pixel groups per warp step
 constexpr int kBandPixels = 2048;    // pixels of a CTA's segment
@@ -173,17 +173,17 @@ __global__ void rect_argmax_kernel(const unsigned long long *counts, int n, int 
 
 using namespace ctm;
 
-// Census of rows [y0, y1) of an image (clipped to it): of the part of the image their
-// windows read, which starts at an even row, so that its rows stay word-aligned.  Rows of
-// that part outside [y0, y1) get codes no one reads.
-static cudaError_t census_rows(const ctm_params &p, const uint8_t *img, int width, int height, int pitch, long long y0,
-                               long long y1, uint64_t *codes, cudaStream_t s)
+// The part of an image that the census of its rows [y0, y1) (clipped to it) reads: it
+// starts at an even row, so that its rows stay word-aligned.  Rows of that part outside
+// [y0, y1) get codes no one reads.  False: no rows.
+static bool census_part(const ctm_params &p, const uint8_t *img, int width, int height, int pitch, long long y0,
+                        long long y1, uint64_t *codes, ctm::CensusImage *part)
 {
     const int sy = p.win_h / 2;
     const long long a = std::max(y0 - sy, 0ll) & ~1ll, b = std::min(y1 + sy, (long long)height);
-    if (b <= a) return cudaSuccess;
-    return launch_census_single(img + a * pitch, width, (int)(b - a), pitch, 1, p.win_w, p.win_h, p.sentinel,
-                                codes + a * width, width, s);
+    if (b <= a) return false;
+    *part = ctm::CensusImage{img + a * pitch, width, (int)(b - a), codes + a * width};
+    return true;
 }
 
 extern "C" int ctm_auto_rect(const ctm_params *p, const uint8_t *left_dev, const uint8_t *right_dev, int width,
@@ -209,8 +209,12 @@ extern "C" int ctm_auto_rect(const ctm_params *p, const uint8_t *left_dev, const
     cudaError_t e = cudaMemsetAsync(counts_dev, 0, sizeof(unsigned long long) * nd, s);
     if (e == cudaSuccess && rx1 > rx0 && ry1 > ry0) {
         // the rows the search reads: the ROI's on the right, moved by every offset on the left
-        e = census_rows(*p, left_dev, width, height, pitch, (long long)ry0 + delta_min, (long long)ry1 + delta_max, CL, s);
-        if (e == cudaSuccess) e = census_rows(*p, right_dev, width, height, pitch, ry0, ry1, CR, s);
+        CensusImage parts[2];
+        int n = 0;
+        n += census_part(*p, left_dev, width, height, pitch, (long long)ry0 + delta_min, (long long)ry1 + delta_max, CL,
+                         parts + n);
+        n += census_part(*p, right_dev, width, height, pitch, ry0, ry1, CR, parts + n);
+        if (n > 0) e = launch_census_images(parts, n, pitch, 1, p->win_w, p->win_h, p->sentinel, cpitch, s);
         const int ndisp = dmax - dmin + 1, w = rx1 - rx0;
         // one band of costs for both searches where the pixels are wide enough against the
         // nd - 1 pixels it adds on both sides: (w + 2 nd) nd costs against 2 w nd, equal at
