@@ -56,17 +56,17 @@ POPC_PER_EVAL = 2          # one u64 code pair = two 32-bit popcounts
 # count was taken.  When the sources differ, or no count was taken, traffic is reported as
 # null.
 TRAFFIC = {
-    # match_persistent_kernel: 118.189 MB read + 1.353 MB written
-    "match": {"bytes": 119.5423e6, "sha": "1f4c15893fcc",
-              "sources": ("match.cu", "match_common.cuh", "aggregate.cuh", "ctm_internal.cuh")},
-    # census_roi4_kernel (60.943 MB read + 63.234 MB written) + tile_list_kernel (0.776 MB)
-    "census": {"bytes": 124.9526e6, "sha": "eb9a08632673",
+    # match_tc_kernel: 116.082 MB read + 2.939 MB written
+    "match": {"bytes": 119.0208e6, "sha": "1c90f400a2b8",
+              "sources": ("match_tc.cu", "match_common.cuh", "aggregate.cuh", "ctm_internal.cuh")},
+    # census_unit_kernel (61.046 MB read + 86.615 MB written) + unit_list_kernel (0.776 MB)
+    "census": {"bytes": 148.4368e6, "sha": "70bb9a7861e3",
                "sources": ("census.cu", "ctm_internal.cuh")},
 }
 CENSUS_TILE_PX = 32        # pixels per listed census tile
-# kernels of one step of the batched path (ctm_box_points, timed apart, is not in it): plan,
-# sample (with census demand marking), tile_list, census_roi, match, aggregate
-KERNELS_PER_STEP = 6
+# kernels of one step of the batched path (ctm_box_points, timed apart, is not in it): plan
+# (with sampling and census demand marking), census list, census, match, aggregate
+KERNELS_PER_STEP = 5
 
 
 def parse():
@@ -772,7 +772,9 @@ def main():
         ncodes = (-(-W // k)) * (-(-H // k))
         census_full[f"k{k}"] = {"ms": cms, "codes": ncodes, "GB_s": 9 * ncodes / (cms * 1e-3) / 1e9}
 
-    # ---- roofline of the matching kernel (integer popcount pipe)
+    # ---- roofline of the matching kernel against the integer popcount pipe (what an xor and two
+    # popcounts per evaluation would be held by; the tensor-core matcher computes the same
+    # evaluations as products and is held by issue slots)
     sms = torch.cuda.get_device_properties(local_rank).multi_processor_count
     popc_rate = B.probe_int_rate(0, 4096)
     popc_clk = float(round(popc_rate))
@@ -797,18 +799,17 @@ def main():
             hbm_peak = float(mp["hbm_gbs"])
             hbm_basis = "of measured copy bandwidth (MEASURED_PEAKS.json)"
 
-    # ---- census phase (tile list + ROI census): HBM and integer-ALU fractions.  Algorithmic
-    # bytes per code: 8 written + 1 source pixel read; compares per code: win_w * win_h - 1,
-    # each half an IMAD (FMA pipe) and half a LOP3 (ALU pipe), the two pipes running side by side
+    # ---- census phase (unit list + ROI census): HBM and integer-ALU fractions.  Algorithmic
+    # bytes per code: 8 written + 1 source pixel read; compares per code: win_w * win_h - 1, 32 of
+    # them eight LOP3 on the ALU pipe (the bit planes and transposes around them are not counted)
     codes = tiles_per_launch * CENSUS_TILE_PX
     n_cmps = w.params["win_w"] * w.params["win_h"] - 1  # compares per code (the centre bit is always 0)
     lop3_rate = B.probe_int_rate(1, 4096)
-    imad_rate = B.probe_int_rate(4, 4096)
-    cmp_clk = min(lop3_rate, imad_rate) / 0.5
+    cmp_clk = lop3_rate * 32 / 8
     cmp_peak = sms * cmp_clk * SM_MAX_MHZ * 1e6 / 1e12
     census_bytes = codes * 9
     census_roof = {
-        "kernel": "tile_list_kernel + census_roi4_kernel (census phase)",
+        "kernel": "unit_list_kernel + census_unit_kernel (census phase)",
         "codes_per_step": codes,
         "hbm": {"achieved": census_bytes / (census_ms * 1e-3) / 1e9, "peak": hbm_peak, "unit": "GB/s",
                 "frac": census_bytes / (census_ms * 1e-3) / 1e9 / hbm_peak,
@@ -817,7 +818,7 @@ def main():
         "alu": {"achieved": codes * n_cmps / (census_ms * 1e-3) / 1e12, "peak": cmp_peak,
                 "unit": "T compares/s", "frac": codes * n_cmps / (census_ms * 1e-3) / 1e12 / cmp_peak,
                 "basis": f"{sms} SMs x {cmp_clk:.0f} compares/clk/SM (LOP3 probe {lop3_rate:.1f}, "
-                         f"IMAD probe {imad_rate:.1f}, one of each per 2 compares) x {SM_MAX_MHZ:g} MHz"},
+                         f"eight per 32 compares) x {SM_MAX_MHZ:g} MHz"},
     }
 
     # ---- the 8 x 3840x2160 workload measured the same way, reported beside the default one
@@ -903,9 +904,11 @@ def main():
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": UNIT,
                          "frac": achieved / peak,
                          "traffic": traffic_bytes("match") if default_workload else None,
-                         "kernel": "match_persistent_kernel",
+                         "kernel": "match_tc_kernel",
                          "peak_basis": f"{sms} SMs x {popc_clk:g} popc32/clk/SM (probe {popc_rate:.2f}) / "
-                                       f"{POPC_PER_EVAL} per eval x {SM_MAX_MHZ:g} MHz",
+                                       f"{POPC_PER_EVAL} per eval x {SM_MAX_MHZ:g} MHz; the kernel computes the same "
+                                       "evaluations as exact e2m1 products on the tensor cores, so the "
+                                       "fraction can pass 1",
                          "at_other_clocks": peak_at},
             "census_roofline": census_roof,
             "batch8x2160": other,
