@@ -397,7 +397,8 @@ int ctm_probe_int_rate(int kind, int iters, double *ops_per_clk_per_sm);
  * tuning match_mode 0; not a graph replay, not the plain per-box path) has its
  * worker that takes the queue's first block withhold the completion signal of
  * that block's products.  The worker's bounded wait then expires (about 1 s, then
- * about 1 s more), it records the error, lets its products end and stops;
+ * about 1 s more), it records the error, waits for no further product of the block,
+ * lets what is in flight end (about 1 s more) and stops;
  * the other workers finish the queue.  The call's outputs follow the CTM_ETIMEOUT
  * rule above, and ctm_match_batch_host returns CTM_ETIMEOUT.  The arming is
  * consumed by that one call; the context stays usable.  No GPU fault is

@@ -79,6 +79,8 @@ struct __align__(128) Shared {
     int next_b;                                  // the next block; -1: none
     int d_f, dy_f;                               // forward match of the block
     int fail;                                    // a bounded wait expired (read after worker_sync)
+    int *err;                                    // the call's error flag
+    int give_up;                                 // the same within a pass: nothing is waited for any more
 };
 
 // Bit planes of a strip code as e2m1 values, 8 words in the order (plane, half).
@@ -229,6 +231,28 @@ __device__ __forceinline__ int strip_stride(int cols) { return (cols + 31) & ~31
 // After worker_sync: a bounded wait of this worker expired.
 __device__ __forceinline__ bool failed(const Shared &sh) { return *reinterpret_cast<const volatile int *>(&sh.fail) != 0; }
 
+// A bounded wait of the worker.  The first that expires ends the waiting of all its
+// warps: the pass keeps up its named barriers to the end, and an expiry costs two seconds
+// once instead of in each of the pass's products (up to 256 offsets x the strip's width).
+// Only a wait that does not succeed at once looks at give_up: the 4K batch's call takes the
+// 288.5 us it took before; with a look per product in every warp 300.0, with the error
+// flag's address handed to each wait 291.1.
+__device__ __noinline__ bool wait_slow(Shared &sh, uint64_t *mbar, unsigned parity)
+{
+    volatile int *stop = &sh.give_up;
+    if (*stop) return false;
+    if (mbar_wait_for(mbar, parity)) return true;
+    *stop = 1;
+    atomicOr(sh.err, 1);
+    mbar_wait_for(mbar, parity);
+    return false;
+}
+
+__device__ __forceinline__ bool wait_worker(Shared &sh, uint64_t *mbar, unsigned parity)
+{
+    return mbar_try_wait(mbar, parity) || wait_slow(sh, mbar, parity);
+}
+
 // ---------------------------------------------------------------- control warp
 
 // Copy the strip of one product -- `cols` columns from `base`, rows Y_m + dy -- into
@@ -300,13 +324,14 @@ __device__ __forceinline__ bool issue_pass(const MatchArgs &a, const BlockGeom &
     const int stages = (g.ny + kStageRows - 1) / kStageRows;
     const uint64_t desc0 = (uint64_t)((smem_addr(sh.points) & 0x3ffff) >> 4) | ((uint64_t)(256 >> 4) << 16) |
                            ((uint64_t)(128 >> 4) << 32) | (1ull << 46);
-    int *err = &a.ws.counts->error;
     bool ok = true, more = true;
     int e = 0, h = 0;
     Tile t = tile_at(g, ps, ps.lo);
 #pragma unroll 1
     while (more) {
-        ok = ok && mbar_wait_bounded(&sh.landed, ph & 1u, err);
+        // one verdict for the warp, whose lanes may see a phase end on both sides of the limit:
+        // what follows elects a lane of all
+        ok = ok && __all_sync(0xffffffffu, wait_worker(sh, &sh.landed, ph & 1u));
         if (ok) ph ^= 1u;
         bar_arrive(bar_id(w, kBarSignal), 160);
         // the product after this one
@@ -338,7 +363,7 @@ __device__ __forceinline__ bool issue_pass(const MatchArgs &a, const BlockGeom &
         // every builder has read the strip
         if (ok && more) issue_strip(a, g, sh, pl, left, t.base + kTcCols * h, min(kTcCols, t.cols - kTcCols * h),
                                     ps.by + ps.bstep * e);
-        ok = ok && mbar_wait_bounded(&sh.done, (ph >> 1) & 1u, err);
+        ok = ok && __all_sync(0xffffffffu, wait_worker(sh, &sh.done, (ph >> 1) & 1u));
         if (ok) ph ^= 2u;
         bar_sync(bar_id(w, kBarSignal), 160);
     }
@@ -389,12 +414,14 @@ __device__ __forceinline__ void control_warp(const MatchArgs &a, Shared &sh, int
         if (failed(sh) || nb < 0) break;
     }
     cp_async_wait_all();
+    __syncwarp();
     if (failed(sh)) {  // what is in flight ends before the CTA's memory is given back
         if (elect_one()) mma_commit(&sh.last);
         __syncwarp();
         mbar_wait_for(&sh.last, 0u);
         mbar_wait_for(&sh.landed, 0u);
         mbar_wait_for(&sh.landed, 1u);
+        __syncwarp();
     }
 }
 
@@ -460,7 +487,7 @@ __device__ __forceinline__ bool build_product(const MatchArgs &a, const BlockGeo
     for (int q = 0; q < stages; ++q) {
         const int st = q & 1;
         // the products of the stage's previous rows are done
-        if (q >= 2) ok = ok && mbar_wait_bounded(&sh.empty[st], ((empty >> st) & 1u) ^ 1u, &a.ws.counts->error);
+        if (q >= 2) ok = ok && wait_worker(sh, &sh.empty[st], ((empty >> st) & 1u) ^ 1u);
         empty ^= 1u << st;
         if (busy) {
             const uint32_t dst = lanes + st * kStageRows * kRowCols;
@@ -629,7 +656,8 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) match_tc_kernel(MatchArgs
         if (lane == 2) mbar_init(&sh.done, 1);
         if (lane == 3) mbar_init(&sh.landed, 1);
         if (lane == 4) mbar_init(&sh.last, 1);
-        if (lane == 5) sh.fail = 0;
+        if (lane == 5) sh.fail = sh.give_up = 0;
+        if (lane == 6) sh.err = &a.ws.counts->error;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         cp_async_wait_all();
         __syncwarp();
