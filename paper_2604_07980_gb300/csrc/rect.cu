@@ -83,6 +83,20 @@ constexpr int kBandThreads = 256;
 constexpr int kBandGroups = 2;       // 32-pixel groups per warp step
 constexpr int kBandPixels = 2048;    // pixels of a CTA's segment
 
+// The band is taken where a segment holds three ranges of disparities.
+constexpr int kBandRatio = 3;
+
+// Shared memory of a segment of w pixels.
+constexpr size_t band_smem_bytes(int w, int ndisp)
+{
+    return (size_t)12 * (w + 3 * ndisp + 32 * kBandGroups) + sizeof(unsigned) * (size_t)w;
+}
+// of the widest segment and the longest range it is taken for: the limit every call sets,
+// so that no call's is below what another thread's launch needs
+constexpr size_t kBandSmemMax = band_smem_bytes(kBandPixels, kBandPixels / kBandRatio);
+static_assert(kBandSmemMax <= 227 * 1024, "shared memory of a CTA");
+static_assert(sizeof(uint64_t) * (2 * kRectThreads + 3 * 1024) <= 48 * 1024, "rect_kernel needs no raised limit");
+
 __global__ void __launch_bounds__(kBandThreads) rect_band_kernel(const uint64_t *CL, const uint64_t *CR,
                                                                  long long pitch, int W, int H, int sx, int sy,
                                                                  int rx0, int rx1, int ry0, int dmin, int dmax,
@@ -219,11 +233,10 @@ extern "C" int ctm_auto_rect(const ctm_params *p, const uint8_t *left_dev, const
         // one band of costs for both searches where the pixels are wide enough against the
         // nd - 1 pixels it adds on both sides: (w + 2 nd) nd costs against 2 w nd, equal at
         // two ranges, so from three on
-        if (e == cudaSuccess && std::min(w, kBandPixels) >= 3 * ndisp) {
+        if (e == cudaSuccess && std::min(w, kBandPixels) >= kBandRatio * ndisp) {
             const dim3 grid((w + kBandPixels - 1) / kBandPixels, ry1 - ry0, nd);
-            const int n_l = std::min(w, kBandPixels) + 2 * ndisp + 32 * kBandGroups, n_r = n_l + ndisp;
-            const size_t smem = (size_t)12 * n_r + sizeof(unsigned) * (size_t)std::min(w, kBandPixels);
-            e = cudaFuncSetAttribute(rect_band_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            const size_t smem = band_smem_bytes(std::min(w, kBandPixels), ndisp);
+            e = cudaFuncSetAttribute(rect_band_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandSmemMax);
             if (e == cudaSuccess)
                 rect_band_kernel<<<grid, kBandThreads, smem, s>>>(CL, CR, cpitch, width, height, p->win_w / 2,
                                                                   p->win_h / 2, rx0, rx1, ry0, dmin, dmax, delta_min,
@@ -231,11 +244,9 @@ extern "C" int ctm_auto_rect(const ctm_params *p, const uint8_t *left_dev, const
         } else if (e == cudaSuccess) {
             const dim3 grid((w + kRectThreads - 1) / kRectThreads, ry1 - ry0, nd);
             const size_t smem = sizeof(uint64_t) * (size_t)(2 * kRectThreads + 3 * ndisp);
-            e = cudaFuncSetAttribute(rect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e == cudaSuccess)
-                rect_kernel<<<grid, kRectThreads, smem, s>>>(CL, CR, cpitch, width, height, p->win_w / 2, p->win_h / 2,
-                                                             rx0, rx1, ry0, dmin, dmax, delta_min, d_thresh, fb_tol,
-                                                             counts_dev);
+            rect_kernel<<<grid, kRectThreads, smem, s>>>(CL, CR, cpitch, width, height, p->win_w / 2, p->win_h / 2,
+                                                         rx0, rx1, ry0, dmin, dmax, delta_min, d_thresh, fb_tol,
+                                                         counts_dev);
         }
         e = e == cudaSuccess ? cudaGetLastError() : e;
     }
