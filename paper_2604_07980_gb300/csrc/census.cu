@@ -590,8 +590,12 @@ struct PlanePair {
     PlaneDesc d[2];
 };
 
+// planes is indexed where it lies: without __grid_constant__ every thread copies it to
+// local memory first (112 bytes of stack).  Images in a row, without and with it: 1920x1200
+// 10.4 -> 9.6 us, 3840x2160 29.8 -> 27.0, 3839x2159 at half resolution 11.9 -> 11.5.
 template <int WW, int WH>
-__global__ void __launch_bounds__(kFullThreads, kFullCtas) census_full_unit_kernel(PlanePair planes, int sentinel)
+__global__ void __launch_bounds__(kFullThreads, kFullCtas)
+    census_full_unit_kernel(const __grid_constant__ PlanePair planes, int sentinel)
 {
     const PlaneDesc &d = planes.d[blockIdx.z];  // one image, or two in one launch
     __shared__ FullSmem<WH> smem[kFullThreads / 32];
