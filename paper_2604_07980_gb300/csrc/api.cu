@@ -56,13 +56,13 @@ struct ctm_ctx {
     cudaStream_t capture_stream = nullptr;
     cudaGraphExec_t gexec = nullptr;
     GraphKey gkey{};
-    // single-frame graph (ctm_match_boxes from its second call on): its first and last
-    // nodes, the planner and the aggregation, take each call's arguments
+    // single-frame graph (ctm_match_boxes), built with the context and after a change of its
+    // tuning; null if it could not be built.  Its first and last nodes, the planner and the
+    // aggregation, take each call's arguments
     cudaGraph_t sgraph = nullptr;
     cudaGraphExec_t sexec = nullptr;
     cudaGraphNode_t splan = nullptr, sagg = nullptr;
     cudaKernelNodeParams splan_kp{}, sagg_kp{};
-    int single_calls = 0;    // -1: the graph could not be built
     // host end-to-end staging (allocated on first use)
     uint8_t *img_dev = nullptr;
     long long img_pitch = 0;
@@ -254,14 +254,18 @@ struct RelaxedCapture {
 
 // Capture the launches of a single-frame call.  They form a chain: the first node
 // (plan_kernel) and the last (aggregate_kernel) are the only ones that read the caller's
-// pointers, so later calls set those two nodes' arguments.  False if it cannot be built.
-bool build_single_graph(ctm_ctx *ctx, const MatchArgs &a, int grid)
+// pointers, so calls set those two nodes' arguments.  Without the graph calls launch
+// directly.  Built and uploaded here, not by a call: it took the second call of a context
+// 88 us of host time instead of 40.
+void build_single_graph(ctm_ctx *ctx)
 {
+    RelaxedCapture relaxed;
+    const MatchArgs a = make_args(ctx, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
     if (cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return;
     }
-    const int r = enqueue_match(ctx, a, 1, grid, ctx->capture_stream, false, 0, false);
+    const int r = enqueue_match(ctx, a, 1, ctx->sm_count * ctx->ctas_per_sm, ctx->capture_stream, false, 0, false);
     cudaError_t e = cudaStreamEndCapture(ctx->capture_stream, &ctx->sgraph);
     bool ok = r == CTM_OK && e == cudaSuccess && ctx->sgraph;
     size_t n = 1;
@@ -277,12 +281,11 @@ bool build_single_graph(ctm_ctx *ctx, const MatchArgs &a, int grid)
     ok = ok && ctx->sagg != ctx->splan && cudaGraphKernelNodeGetParams(ctx->splan, &ctx->splan_kp) == cudaSuccess &&
          cudaGraphKernelNodeGetParams(ctx->sagg, &ctx->sagg_kp) == cudaSuccess &&
          cudaGraphInstantiate(&ctx->sexec, ctx->sgraph, 0) == cudaSuccess;
-    if (!ok) {
-        ctx->sexec = nullptr;
+    if (!ok) ctx->sexec = nullptr;
+    if (!ok || cudaGraphUpload(ctx->sexec, ctx->capture_stream) != cudaSuccess) {
         drop_single_graph(ctx);
         cudaGetLastError();
     }
-    return ok;
 }
 
 int set_device(const ctm_ctx *ctx)
@@ -470,6 +473,7 @@ int ctm_create(ctm_ctx **out, const ctm_params *p, int max_frames, int max_width
         return CTM_ECUDA;
     }
     census_roi_ctas_per_sm(p->win_w, p->win_h);  // outside any capture
+    build_single_graph(ctx);
     *out = ctx;
     return CTM_OK;
 }
@@ -536,24 +540,17 @@ int ctm_match_boxes(ctm_ctx *ctx, const uint8_t *left_dev, const uint8_t *right_
     const int slots = std::max(1, ctx->p.grid_g * ctx->p.grid_g);
     const long long blocks_ub = (long long)std::max(n_boxes, 1) * slots;
     const int grid = (int)std::min<long long>((long long)ctx->sm_count * ctx->ctas_per_sm, blocks_ub);
-    // From the second call on the launches replay as a graph (one submission and two
-    // argument updates instead of seven launches: a call of four boxes 0.063 -> 0.041 ms in a
-    // row); not for diagnostics, an armed fault injection or a stream being captured.
+    // The launches replay as a graph (one submission and two argument updates instead of
+    // five launches: a call of four boxes 0.063 -> 0.041 ms in a row, when it was seven);
+    // not for diagnostics, an armed fault injection or a stream being captured.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    bool replay = ctx->single_calls > 0 && !dbg && !ctx->inject_expiry;
+    bool replay = ctx->sexec && !dbg && !ctx->inject_expiry;
     RelaxedCapture relaxed;
     if (replay && (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)) {
         cudaGetLastError();
         replay = false;
     }
-    if (replay && !ctx->sexec && !build_single_graph(ctx, a, ctx->sm_count * ctx->ctas_per_sm)) {
-        ctx->single_calls = -1;
-        replay = false;
-    }
-    if (!replay) {
-        if (ctx->single_calls == 0) ctx->single_calls = 1;
-        return enqueue_match(ctx, a, 1, grid, s, false, n_boxes);
-    }
+    if (!replay) return enqueue_match(ctx, a, 1, grid, s, false, n_boxes);
     a.caps.max_frames = 1;
     cudaKernelNodeParams kp = ctx->splan_kp;
     void *plan_args[2] = {&a, ctx->splan_kp.kernelParams[1]};
@@ -1016,6 +1013,7 @@ int ctm_set_tuning(ctm_ctx *ctx, const ctm_tuning *t)
         if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
         ctx->gexec = nullptr;
         drop_single_graph(ctx);
+        build_single_graph(ctx);
     }
     return CTM_OK;
 }
