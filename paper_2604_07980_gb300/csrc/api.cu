@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "ctm_internal.cuh"
+#include "host_tables.h"
 
 using namespace ctm;
 
@@ -66,15 +67,9 @@ struct ctm_ctx {
     // host end-to-end staging (allocated on first use)
     uint8_t *img_dev = nullptr;
     long long img_pitch = 0;
-    ctm_box *boxes_dev = nullptr;
-    // tables of a host call -- counts, frames, boxes, copied together -- and its results
-    // (disparities, depths, flags one behind the other), in device and page-locked memory
+    // tables of a host call -- counts, frames, boxes (host_tables.h), copied together -- and its
+    // results (disparities, depths, flags one behind the other), in device and page-locked memory
     char *tables_dev = nullptr, *tables_host = nullptr, *results_dev = nullptr, *results_host = nullptr;
-    ctm_frame *frames_host_pinned = nullptr;
-    int32_t *counts_host_pinned = nullptr;
-    ctm_box *boxes_host_pinned = nullptr;
-    ctm_frame *frames_dev2 = nullptr;
-    int32_t *counts_dev2 = nullptr;
     cudaStream_t copy_stream = nullptr;         // host-to-device copies of the sub-batches
     cudaEvent_t host_ev[kHostGroups + 1] = {};  // sub-batch g copied; [kHostGroups]: start
 };
@@ -672,19 +667,19 @@ int ctm_match_batch_profiled(ctm_ctx *ctx, const ctm_frame *frames_dev, const in
 }
 
 // Staging of the host entry points (allocated on first use): device images at
-// a pitch of 128 bytes; per sub-batch counts, two frame tables (the staging images'
-// and, for mapped calls, the caller's) and boxes, in that order; results; the same two
+// a pitch of 128 bytes; the call's tables (per sub-batch counts, the staging images' frame
+// table and, for mapped calls, the caller's, boxes: host_tables.h); results; the same two
 // blocks in page-locked memory; a copy stream and its events.
-constexpr size_t kTablesFrames = 256;  // offset of the frame tables, after 4 kHostGroups counts
-static_assert(sizeof(int32_t) * 4 * kHostGroups <= kTablesFrames, "counts of the sub-batches");
+static_assert(sizeof(int32_t) * 4 * kHostGroups <= kHostCountsBytes, "counts of the sub-batches");
 
 static int ensure_host_staging(ctm_ctx *ctx)
 {
     if (ctx->img_dev) return CTM_OK;
     ctx->img_pitch = round_up(ctx->caps.max_width, 128);
     const size_t img_bytes = (size_t)round_up((long long)ctx->img_pitch * ctx->caps.max_height * 2 * ctx->caps.max_frames, 256);
-    const size_t o_boxes = kTablesFrames + (size_t)round_up((long long)(sizeof(ctm_frame) * 2 * ctx->caps.max_frames), 256);
-    const size_t tables = (size_t)round_up((long long)(o_boxes + sizeof(ctm_box) * (size_t)ctx->caps.max_boxes), 256);
+    const size_t nf = (size_t)ctx->caps.max_frames;
+    const HostTables cap = host_tables(nf, nf, (size_t)ctx->caps.max_boxes, sizeof(ctm_frame), sizeof(ctm_box));
+    const size_t tables = (size_t)round_up((long long)cap.bytes, 256);
     const size_t results = 9 * (size_t)ctx->caps.max_boxes;  // two floats and a byte each
     void *mem = nullptr;
     if (dev_alloc(&mem, img_bytes + tables + results) != cudaSuccess) { cudaGetLastError(); return CTM_ENOMEM; }
@@ -708,23 +703,29 @@ static int ensure_host_staging(ctm_ctx *ctx)
     ctx->tables_dev = b + img_bytes;
     ctx->results_dev = ctx->tables_dev + tables;
     ctx->results_host = ctx->tables_host + tables;
-    ctx->counts_dev2 = reinterpret_cast<int32_t *>(ctx->tables_dev);
-    ctx->frames_dev2 = reinterpret_cast<ctm_frame *>(ctx->tables_dev + kTablesFrames);
-    ctx->boxes_dev = reinterpret_cast<ctm_box *>(ctx->tables_dev + o_boxes);
-    ctx->counts_host_pinned = reinterpret_cast<int32_t *>(ctx->tables_host);
-    ctx->frames_host_pinned = reinterpret_cast<ctm_frame *>(ctx->tables_host + kTablesFrames);
-    ctx->boxes_host_pinned = reinterpret_cast<ctm_box *>(ctx->tables_host + o_boxes);
     return CTM_OK;
+}
+
+// A call's tables in one of the two blocks.
+struct Tables {
+    int32_t *counts;
+    ctm_frame *frames, *sources;
+    ctm_box *boxes;
+};
+
+static Tables tables_at(char *base, const HostTables &t)
+{
+    return Tables{reinterpret_cast<int32_t *>(base), reinterpret_cast<ctm_frame *>(base + t.frames),
+                  reinterpret_cast<ctm_frame *>(base + t.sources), reinterpret_cast<ctm_box *>(base + t.boxes)};
 }
 
 // Counts, frames and the call's boxes in one copy (four copies of a few KB each took
 // about 2 us of the host apiece).
-static cudaError_t copy_tables(ctm_ctx *ctx, const ctm_box *boxes_host, int n_boxes, cudaStream_t s)
+static cudaError_t copy_tables(ctm_ctx *ctx, const HostTables &t, const ctm_box *boxes_host, int n_boxes,
+                               cudaStream_t s)
 {
-    if (n_boxes > 0) memcpy(ctx->boxes_host_pinned, boxes_host, sizeof(ctm_box) * (size_t)n_boxes);
-    const size_t bytes = (size_t)(reinterpret_cast<char *>(ctx->boxes_host_pinned) - ctx->tables_host) +
-                         sizeof(ctm_box) * (size_t)n_boxes;
-    return cudaMemcpyAsync(ctx->tables_dev, ctx->tables_host, bytes, cudaMemcpyHostToDevice, s);
+    if (n_boxes > 0) memcpy(ctx->tables_host + t.boxes, boxes_host, sizeof(ctm_box) * (size_t)n_boxes);
+    return cudaMemcpyAsync(ctx->tables_dev, ctx->tables_host, t.bytes, cudaMemcpyHostToDevice, s);
 }
 
 // Where a host call's kernels put their results: n floats, n floats, n bytes.
@@ -749,7 +750,7 @@ static int host_results(ctm_ctx *ctx, cudaStream_t s, int n_boxes, float *disp_h
     cudaError_t e = cudaSuccess;
     if (n_boxes > 0)
         e = cudaMemcpyAsync(ctx->results_host, ctx->results_dev, 9 * (size_t)n_boxes, cudaMemcpyDeviceToHost, s);
-    int32_t *err_h = ctx->counts_host_pinned + 4 * kHostGroups - 1;  // a slot no sub-batch uses
+    int32_t *err_h = reinterpret_cast<int32_t *>(ctx->tables_host) + 4 * kHostGroups - 1;  // a slot no sub-batch uses
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(err_h, &ctx->ws.stats->error, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -858,6 +859,8 @@ int ctm_match_batch_host(ctm_ctx *ctx, const ctm_frame *frames_host, int n_frame
         if (n_frames < 2 * groups) return (int)((long long)g * n_frames / groups);
         return (int)(((long long)k64ths[groups - 1][g] * n_frames + 32) / 64);
     };
+    const HostTables lay = host_tables((size_t)n_frames, 0, (size_t)n_boxes, sizeof(ctm_frame), sizeof(ctm_box));
+    const Tables host = tables_at(ctx->tables_host, lay), dev = tables_at(ctx->tables_dev, lay);
     // every sub-batch's tables ahead of the images
     for (int g = 0; g < groups; ++g) {
         const int f0 = bound(g), f1 = bound(g + 1);
@@ -868,13 +871,13 @@ int ctm_match_batch_host(ctm_ctx *ctx, const ctm_frame *frames_host, int n_frame
             t.right = t.left + plane;
             t.pitch = (int32_t)ctx->img_pitch;
             t.box_begin -= box0;
-            ctx->frames_host_pinned[i] = t;
+            host.frames[i] = t;
         }
-        ctx->counts_host_pinned[4 * g] = f1 - f0;
-        ctx->counts_host_pinned[4 * g + 1] =
+        host.counts[4 * g] = f1 - f0;
+        host.counts[4 * g + 1] =
             groups > 1 ? frames_host[f1 - 1].box_begin + frames_host[f1 - 1].box_count - box0 : n_boxes;
     }
-    if (e == cudaSuccess) e = copy_tables(ctx, boxes_host, n_boxes, cs);
+    if (e == cudaSuccess) e = copy_tables(ctx, lay, boxes_host, n_boxes, cs);
     const HostResults res = host_results_at(ctx->results_dev, n_boxes);
     for (int g = 0; g < groups && e == cudaSuccess; ++g) {
         const int f0 = bound(g), f1 = bound(g + 1);
@@ -889,7 +892,7 @@ int ctm_match_batch_host(ctm_ctx *ctx, const ctm_frame *frames_host, int n_frame
         if (e == cudaSuccess) e = cudaEventRecord(ctx->host_ev[g], cs);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ctx->host_ev[g], 0);
         if (e != cudaSuccess) break;
-        MatchArgs a = make_args(ctx, ctx->frames_dev2 + f0, ctx->counts_dev2 + 4 * g, ctx->boxes_dev + box0,
+        MatchArgs a = make_args(ctx, dev.frames + f0, dev.counts + 4 * g, dev.boxes + box0,
                                 res.disp + box0, res.depth + box0, res.flags + box0, nullptr);
         a.stats_accumulate = g > 0;  // ctm_get_stats then covers the whole call
         if (enqueue_match(ctx, a, f1 - f0, grid, s, false, 0) != CTM_OK) e = cudaErrorLaunchFailure;
@@ -915,12 +918,14 @@ int ctm_match_batch_mapped(ctm_ctx *ctx, const ctm_frame *frames_host, int n_fra
     cudaStream_t s = (cudaStream_t)stream;
     st = ensure_host_staging(ctx);
     if (st != CTM_OK) return st;
-    // the staging images' frame table and the caller's (second half of the tables); a
-    // frame the gather cannot read in place (rows or width off 16-byte multiples, or
-    // memory the device cannot read at its host address) is copied whole on s and gets
-    // height 0 in the gather's table
+    // the staging images' frame table and the caller's; a frame the gather cannot read in
+    // place (rows or width off 16-byte multiples, or memory the device cannot read at its
+    // host address) is copied whole on s and gets height 0 in the gather's table
     const size_t plane = (size_t)ctx->img_pitch * ctx->caps.max_height;
-    ctm_frame *stage = ctx->frames_host_pinned, *src = ctx->frames_host_pinned + ctx->caps.max_frames;
+    const HostTables lay =
+        host_tables((size_t)n_frames, (size_t)n_frames, (size_t)n_boxes, sizeof(ctm_frame), sizeof(ctm_box));
+    const Tables host = tables_at(ctx->tables_host, lay), dev = tables_at(ctx->tables_dev, lay);
+    ctm_frame *stage = host.frames, *src = host.sources;
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < n_frames && e == cudaSuccess; ++i) {
         const ctm_frame &f = frames_host[i];
@@ -941,15 +946,13 @@ int ctm_match_batch_mapped(ctm_ctx *ctx, const ctm_frame *frames_host, int n_fra
                                       f.height, cudaMemcpyHostToDevice, s);
         }
     }
-    int32_t *cnt = ctx->counts_host_pinned;
-    cnt[0] = n_frames;
-    cnt[1] = n_boxes;
-    if (e == cudaSuccess) e = copy_tables(ctx, boxes_host, n_boxes, s);
+    host.counts[0] = n_frames;
+    host.counts[1] = n_boxes;
+    if (e == cudaSuccess) e = copy_tables(ctx, lay, boxes_host, n_boxes, s);
     if (e == cudaSuccess) {
         const HostResults res = host_results_at(ctx->results_dev, n_boxes);
-        MatchArgs a = make_args(ctx, ctx->frames_dev2, ctx->counts_dev2, ctx->boxes_dev, res.disp, res.depth,
-                                res.flags, nullptr);
-        a.gather_src = ctx->frames_dev2 + ctx->caps.max_frames;
+        MatchArgs a = make_args(ctx, dev.frames, dev.counts, dev.boxes, res.disp, res.depth, res.flags, nullptr);
+        a.gather_src = dev.sources;
         const int grid = ctx->sm_count * ctx->ctas_per_sm;
         if (enqueue_match(ctx, a, n_frames, grid, s, false, 0) != CTM_OK) e = cudaErrorLaunchFailure;
     }
