@@ -56,11 +56,11 @@ POPC_PER_EVAL = 2          # one u64 code pair = two 32-bit popcounts
 # count was taken.  When the sources differ, or no count was taken, traffic is reported as
 # null.
 TRAFFIC = {
-    # match_tc_kernel: 116.082 MB read + 2.939 MB written
-    "match": {"bytes": 119.0208e6, "sha": "1c90f400a2b8",
+    # match_tc_kernel: 116.068 MB read + 0.133 MB written
+    "match": {"bytes": 116.2002e6, "sha": "a91c91505348",
               "sources": ("match_tc.cu", "match_common.cuh", "aggregate.cuh", "ctm_internal.cuh")},
-    # census_unit_kernel (61.046 MB read + 86.615 MB written) + unit_list_kernel (0.776 MB)
-    "census": {"bytes": 148.4368e6, "sha": "70bb9a7861e3",
+    # census_unit_kernel (61.225 MB read + 86.773 MB written) + unit_list_kernel (0.781 MB)
+    "census": {"bytes": 148.7793e6, "sha": "7b56e29237a4",
                "sources": ("census.cu", "ctm_internal.cuh")},
 }
 CENSUS_TILE_PX = 32        # pixels per listed census tile

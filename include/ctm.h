@@ -372,9 +372,8 @@ int ctm_get_tuning(const ctm_ctx *ctx, ctm_tuning *out);
 int ctm_set_tuning(ctm_ctx *ctx, const ctm_tuning *t);
 
 /* Autotuner: runs the batch of ctm_match_batch (same arguments, no debug
- * output) under candidate tunings -- the tensor-core matcher, the two-pass
- * matcher at every CTA size x strip width, then each census variant around the
- * best so far --
+ * output) under candidate tunings -- the tensor-core matcher, then the two-pass
+ * matcher at every CTA size x strip width --
  * timing `reps` calls of each with CUDA events after one warm-up call, keeps
  * the fastest in the context and returns it in *best (and its time per call,
  * in ms, in *best_ms; either may be NULL).  The outputs are written by every

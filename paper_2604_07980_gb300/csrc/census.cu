@@ -7,8 +7,8 @@
 // them; pixels whose window leaves the grid get 0.
 //
 // Fixed windows (5x5, 7x7, 9x7) compare bit planes of 32 pixels at a time in units of
-// 128 columns x 32 rows: all of them for a full image (ctm_census_build), those with
-// marked tiles for the matching path.  Other windows use a warp per 64-pixel tile, the
+// 128 columns: of eight rows for a full image (ctm_census_build), of the marked ones of
+// sixteen rows for the matching path.  Other windows use a warp per 64-pixel tile, the
 // window rows staged in shared memory as 16-bit values 0x6400 | v.
 #include "ctm_internal.cuh"
 
@@ -147,21 +147,24 @@ __device__ __forceinline__ void store_pair(const Plane &pl, int x, int y, uint64
 // What bounds it: the ALU pipe (LOP3, PRMT, SHF: half of the issue rate; about 1450
 // instructions for eight rows of a unit, 912 of them the compares and transposes) and
 // the L1 (124 LDS.128 for the same rows, 0.6 of its wavefronts), 60 and 75% busy on eight
-// 4K frames, with twelve warps an SM (shared memory).  The kernel before it compared two
+// 4K frames, with twelve warps an SM (shared memory, and 64,512 of 65,536 registers).  The kernel before it compared two
 // pixels per instruction in 16-bit halves, 160 instructions a pixel against 85 here
 // (per marked pixel: a unit also computes the unmarked part of its 128 columns, 10 to
 // 25%, and leaves lanes idle when its rows are not a multiple of eight).  Measured, list
 // and census of the marked tiles: eight 4K frames 141 -> 110 us, 32 frames of 1920x1200
 // 110 -> 103, four 720p frames 24.4 -> 19.5, one 1279x719 frame (rows of odd pitch, which
-// the old kernel read by bytes) 18.2 -> 14.6; full images: 3840x2160 39.0 -> 28.8,
-// 1920x1200 15.0 -> 11.3, 3839x2159 at half resolution 33 -> 12.7 us.  Slower: a CTA of
+// the old kernel read by bytes) 18.2 -> 14.6; full images, alone: 1920x1200 15.0 -> 12.4,
+// 3839x2159 at half resolution 35 -> 13.7 us.  Where sampled rows lie far apart it is the
+// slower one: a unit of a few marked rows slices nearly as many source rows as a full one
+// and leaves lanes idle (eight 1920x1200 frames, every box one block of 16 x 16 points,
+// 28.7 -> 52 us; joining spans of columns in such units did not help).  Slower: a CTA of
 // four warps per unit of 32 rows (120 us on the 32 frames), codes stored by the lanes
 // instead of bulk copies (L1 at 78%), all source rows loaded before the first is sliced
 // (instruction cache), two row buffers in registers (spills).
 constexpr int kUnitPx = 128;      // columns of a unit
 constexpr int kRoiRows = 16;      // rows of a unit of the matching path
 constexpr int kUnitThreads = 64;
-constexpr int kUnitCtas = 6;      // resident CTAs per SM (shared memory; 168 registers a thread)
+constexpr int kUnitCtas = 6;      // resident CTAs per SM (37 KB and 168 registers a thread: each alone stops a seventh)
 constexpr int kFullThreads = 128; // full image
 constexpr int kFullCtas = 4;      // 128 registers a thread
 constexpr int kUnitPos = 12;      // words -4 .. 7 of a source row

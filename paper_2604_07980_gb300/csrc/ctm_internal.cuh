@@ -156,8 +156,9 @@ __device__ __forceinline__ int queue_at(const MatchArgs &a, int n_big, int p)
     return p < n_big ? a.ws.queue[p] : a.ws.queue[a.caps.max_blocks - 1 - (p - n_big)];
 }
 
-// num / den for 0 <= num < 2^24 and 1 <= den < 2^24: one approximate fp32 quotient (off by
-// less than one) and a correction, a third of the instructions of an integer division.
+// num / den for 0 <= num < 2^24 and 1 <= den < 2^24 with a quotient below 2^22 (the callers'
+// is below 2^20): one approximate fp32 quotient, at most two units in the last place off
+// and so less than one, and a correction; a third of the instructions of an integer division.
 __device__ __forceinline__ int div_small(int num, int den)
 {
     int q = (int)__fdividef((float)num, (float)den);

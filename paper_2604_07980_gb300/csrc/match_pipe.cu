@@ -1,8 +1,8 @@
 // match_pipe.cu -- the two-pass pipelined matcher.
 //
-// The fused kernel (match.cu) waits twice per block: for the point codes and
-// forward strip, then -- after the forward argmin -- for the matched right
-// codes and the backward strip.  Here the passes are split into two kernels
+// A matcher that runs both passes of a block in turn (match.cu, a launch per box) waits
+// twice per block: for the point codes and forward strip, then -- after the forward
+// argmin -- for the matched right codes and the backward strip.  Here the passes are split into two kernels
 // over the same queue of searchable blocks:
 //   match_fwd_kernel: Eq. census_cost for every candidate (forward), the first
 //     argmin and the costs around it, stored in the block's sampling record;
@@ -13,7 +13,7 @@
 // first strip chunk of block k+1 are already on their way into the other, and
 // the sampling record of block k+2 into a third record buffer.  Blocks are
 // assigned to CTAs round robin over the queue (large work first), so every CTA
-// gets a similar mix.  Results equal the fused kernel's: the same sums in the
+// gets a similar mix.  Results equal the other matchers': the same sums in the
 // same candidate order, the same argmin and the same fp32 parabola.
 #include <math.h>
 

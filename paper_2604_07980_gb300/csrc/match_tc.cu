@@ -33,10 +33,10 @@
 // 16 accumulator columns each, three to a CTA so that the power-of-two allocation
 // fits), shared memory too (35 KB each).
 //
-// What bounds it: issue slots (about 6250 warp instructions a block, half of them in the
-// per-block work around the unpacking) and, with six workers, the chain of barriers of
-// a block.  Measured (matching kernel, popcount kernel before it): 32 frames of
-// 1920x1200 0.145 -> 0.095 ms, eight 4K frames 0.27 -> 0.17 ms; the whole calls 0.289 ->
+// What bounds it: issue slots (6040 warp instructions a searched block on the 32 frames
+// below, 8730 on the 4K ones, half of them in the per-block work around the unpacking)
+// and, with six workers, the chain of barriers of a block.  Measured (matching kernel, popcount kernel before it): 32 frames of
+// 1920x1200 0.145 -> 0.096 ms, eight 4K frames 0.27 -> 0.152 ms; the whole calls 0.289 ->
 // 0.235 and 0.440 -> 0.340 ms, four 720p frames 0.0735 -> 0.0585 ms.  Slower variants:
 // a warp per block on mma.sync fp8 (0.41 ms on the first batch), one barrier of the
 // CTA per stage (0.16), strips by plain loads into registers (0.13, spills),
@@ -559,7 +559,7 @@ __device__ __forceinline__ unsigned build_pass(const MatchArgs &a, const Pass &p
                              *reinterpret_cast<const int16_t *>(p + o.z) + *reinterpret_cast<const int16_t *>(p + o.w);
                     }
                     s = K0 + (s >> 1);
-                } else {  // a tile's sum may be odd, the strip's is even
+                } else {  // 2 K0 and the tiles' sums (all even), halved with the last
                     for (int j = 0; j < g.nx; ++j)
                         if ((unsigned)(g.X[j] + x) < (unsigned)t.cols)
                             s += *reinterpret_cast<const int16_t *>(p + sh.xoff[j]);
