@@ -206,9 +206,10 @@ int ctm_census_build(const uint8_t *img_dev, int width, int height, int pitch, i
  * (uint8 CTM_BOX_*).  dbg may be NULL.  The launch sequence of the batch path on
  * one frame: device planning and point sampling, the census of the row tiles the
  * search reads (both images, both resolutions), one persistent matching kernel
- * and a per-box aggregation kernel.  The launches replay as a CUDA graph that the
- * context was created with, whose arguments each call sets (not with dbg, nor while
- * `stream` is being captured).  Errors: CTM_EINVAL, CTM_ENOMEM (beyond
+ * and a per-box aggregation kernel.  The launches replay as a CUDA graph that a
+ * context of one frame is created with (else the first call builds it), whose
+ * arguments each call sets (not with dbg, nor while `stream` is being captured).
+ * Errors: CTM_EINVAL, CTM_ENOMEM (beyond
  * capacity), CTM_ECUDA. */
 int ctm_match_boxes(ctm_ctx *ctx, const uint8_t *left_dev, const uint8_t *right_dev,
                     int width, int height, int pitch, const ctm_box *boxes_dev, int n_boxes,
@@ -367,7 +368,7 @@ int ctm_get_tuning(const ctm_ctx *ctx, ctm_tuning *out);
 /* Set the tuning (CTM_EINVAL if a field is out of range or the strip does not
  * fit in shared memory; the context keeps its previous tuning then).  A
  * captured batch graph is dropped and recaptured by the next graph call; the
- * single-frame graph is rebuilt here.
+ * single-frame graph of a context of one frame is rebuilt here.
  * Synchronous; do not call while a stream capture is active. */
 int ctm_set_tuning(ctm_ctx *ctx, const ctm_tuning *t);
 

@@ -57,13 +57,14 @@ struct ctm_ctx {
     cudaStream_t capture_stream = nullptr;
     cudaGraphExec_t gexec = nullptr;
     GraphKey gkey{};
-    // single-frame graph (ctm_match_boxes), built with the context and after a change of its
-    // tuning; null if it could not be built.  Its first and last nodes, the planner and the
-    // aggregation, take each call's arguments
+    // single-frame graph (ctm_match_boxes), built with a context of one frame and after a change
+    // of its tuning, else by the first call; null if it could not be built.  Its first and last
+    // nodes, the planner and the aggregation, take each call's arguments
     cudaGraph_t sgraph = nullptr;
     cudaGraphExec_t sexec = nullptr;
     cudaGraphNode_t splan = nullptr, sagg = nullptr;
     cudaKernelNodeParams splan_kp{}, sagg_kp{};
+    bool single_tried = false;  // built, or found that it cannot be
     // host end-to-end staging (allocated on first use)
     uint8_t *img_dev = nullptr;
     long long img_pitch = 0;
@@ -250,12 +251,14 @@ struct RelaxedCapture {
 // Capture the launches of a single-frame call.  They form a chain: the first node
 // (plan_kernel) and the last (aggregate_kernel) are the only ones that read the caller's
 // pointers, so calls set those two nodes' arguments.  Without the graph calls launch
-// directly.  Built here, not by a call: it took the second call of a context 88 us of
-// host time instead of 40.  Not uploaded: with an uploaded graph in the context, every
-// replay of its batch graph took 1.4 us more.
+// directly.  Built with a context of one frame, not by a call: it took the second call
+// 88 us of host time instead of 40.  A context of several frames is for batches, whose
+// replays take 0.3 us more beside a second graph (1.4 us more once that is uploaded, which
+// is therefore left to its first launch), so there the first single-frame call builds it.
 void build_single_graph(ctm_ctx *ctx)
 {
     RelaxedCapture relaxed;
+    ctx->single_tried = true;
     const MatchArgs a = make_args(ctx, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
     if (cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
         cudaGetLastError();
@@ -469,7 +472,7 @@ int ctm_create(ctm_ctx **out, const ctm_params *p, int max_frames, int max_width
         return CTM_ECUDA;
     }
     census_roi_ctas_per_sm(p->win_w, p->win_h);  // outside any capture
-    build_single_graph(ctx);
+    if (max_frames == 1) build_single_graph(ctx);
     *out = ctx;
     return CTM_OK;
 }
@@ -540,13 +543,14 @@ int ctm_match_boxes(ctm_ctx *ctx, const uint8_t *left_dev, const uint8_t *right_
     // five launches: a call of four boxes 0.063 -> 0.041 ms in a row, when it was seven);
     // not for diagnostics, an armed fault injection or a stream being captured.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    bool replay = ctx->sexec && !dbg && !ctx->inject_expiry;
+    bool replay = (ctx->sexec || !ctx->single_tried) && !dbg && !ctx->inject_expiry;
     RelaxedCapture relaxed;
     if (replay && (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)) {
         cudaGetLastError();
         replay = false;
     }
-    if (!replay) return enqueue_match(ctx, a, 1, grid, s, false, n_boxes);
+    if (replay && !ctx->sexec) build_single_graph(ctx);
+    if (!replay || !ctx->sexec) return enqueue_match(ctx, a, 1, grid, s, false, n_boxes);
     a.caps.max_frames = 1;
     cudaKernelNodeParams kp = ctx->splan_kp;
     void *plan_args[2] = {&a, ctx->splan_kp.kernelParams[1]};
@@ -1017,7 +1021,8 @@ int ctm_set_tuning(ctm_ctx *ctx, const ctm_tuning *t)
         if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
         ctx->gexec = nullptr;
         drop_single_graph(ctx);
-        build_single_graph(ctx);
+        ctx->single_tried = false;
+        if (ctx->caps.max_frames == 1) build_single_graph(ctx);
     }
     return CTM_OK;
 }
